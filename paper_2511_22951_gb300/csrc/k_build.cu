@@ -21,7 +21,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <type_traits>
 
 #include "mdk_internal.cuh"
 
@@ -454,14 +453,6 @@ __device__ __forceinline__ bool stencil_cell(int cd, int sd, int nc, int per, in
   return true;
 }
 
-// Verlet lists (the paper's 3x3x3 cell template), one thread per atom in
-// cell order, so the lanes of a warp share most of their stencil cells.
-// Accepted entries are staged in shared memory (two groups of 8 per thread,
-// written while the other is flushed) and reach HBM as full 32-byte sectors
-// of the list layout.  The candidate loop is branch-free: every candidate is
-// stored into the next slot and the count advances only when it is accepted.
-// Candidates near r_ns, and far atoms (NaN offsets), take the exact FP64 test
-// of the definition.
 __device__ __forceinline__ int image_of(int c, int sd, int nc, int per) {
   if (!per) return 0;
   const int q = c + sd;
@@ -496,8 +487,6 @@ __device__ __forceinline__ bool half_keep(int i, int j, bool s_pos) {
   return (i < j) == (((i ^ j) & 1) == 0);
 }
 
-// HALF: the list kind is a template parameter, so a full list's candidate
-// loop carries no half-list test
 // where a build writes: the Verlet list (s.nbr), or with the outer list on
 // the outer list (s.nbr1, radius rc + skin_outer, always full)
 struct ListOut {
@@ -505,118 +494,304 @@ struct ListOut {
   int32_t *nnbr;
   int nmax;
   double rns2;
-  float lo, hi;
   int *max_seen;
 };
 
+// Verlet lists (the paper's 3x3x3 cell template): one warp per slice of at
+// most 32 atoms of one cell, lanes over candidates.
+//
+// The candidates of a cell are its 27 template cells' atoms in template order,
+// flattened: candidate p sits in the range whose cumulative length passes p,
+// so every chunk of 32 candidates is full whatever the cells hold.  Phase 1:
+// lane l loads candidate p (cells are contiguous runs of atoms), shifts it by
+// its stencil offset and tests it against every atom of the slice,
+//   r^2 - r_ns^2 = (c.c - r_ns^2) + p.p - 2 c.p,
+// two atoms per packed FP32 instruction with their constants broadcast from
+// shared memory; one ballot per atom and chunk is that atom's acceptance mask.
+// Phase 2: lane k walks atom k's nonzero mask words bit by bit, one entry per
+// step in every lane (the atoms of a cell have about equally many), and
+// writes them from registers in groups of 8 (full sectors of the list
+// layout).  Candidates sit in the lanes in descending order, so that the
+// next one is the highest set bit (one instruction).
+//
+// What binds it is instruction issue: ~6 instructions per 32 tests, ~30 per
+// 32 candidates loaded and ~15 per step of phase 2.  The version before gave
+// each atom a thread that walked the candidates and staged each of them: 43
+// instructions per candidate (tails of every cell's run, the stencil
+// arithmetic per atom and cell, one shared store per candidate, lanes of two
+// cells diverging).  Phase 2 with a lane per mask word and a scan of their bit
+// counts was slower: the accepted candidates sit in few, dense words.
+// Measured (ncu, one launch, before -> now): 388,204 argon atoms (529 candidates,
+// 78 neighbours) 305 -> 213 us (653 -> 335 warp instructions per atom, issue
+// active 77% -> 55%: the two phases' shared-memory chains take turns with
+// the packed tests); 8,388,608 atoms with the outer list (890 candidates, 136
+// entries) 9.1 -> 6.0 ms; 256 atoms 57 -> 21 us, 32,000 71 -> 46 us.
+//
+// Error of the FP32 test: atoms in their cells (|p_d| <= 0.6 h) give |c| <=
+// 2.8 h, each product and sum rounds to 2^-24 of at most 15 h^2, so r^2 is off
+// by less than 5e-6 h^2; atoms clamped into an end cell of a free dimension
+// (|p_d| <= 2 h) give 75 h^2 and 2.5e-5 h^2.  Candidates within a band four
+// times that wide (Sys.build_band = 2e-5 h^2, and five times it) take the
+// exact FP64 test of the definition, and so do far atoms (NaN offsets).
+// Lists come out in the order of the candidates: template cell, then atom.
+constexpr int kBWarps = 4;     // warps per block
+constexpr int kTileCh = 32;    // chunks of 32 candidates per tile (two phases per tile)
+// Atoms of a slice at most, by the size of the system: short slices give a
+// small system more warps (a warp's chain of dependent loads and shared
+// reads takes ~10 us whatever its slice holds), long ones share the loading
+// of the candidates.  k_build in us with 8 / 16 / 32 atoms per slice: 256 LJ
+// atoms 21 / 24 / 29, 9,724 EAM 32 / 36 / 50, 32,000 LJ 57 / 46 / 58, 131,072
+// (6 A lists) 141 / 106 / 95, 388,204 LJ 412 / 297 / 213.
+inline int slice_atoms(int n) { return n < 16384 ? 8 : (n < 65536 ? 16 : 32); }
+struct BuildWarp {
+  uint32_t ent[kTileCh * 32];      // list entries of the tile's candidates, by chunk and lane
+  uint4 mask[kTileCh / 2][16];     // per chunk and atom pair: (c, k), (c, k+1), (c+1, k), (c+1, k+1)
+  float4 a0[16], a1[16];           // atom pairs: -2x, -2x', -2y, -2y' | -2z, -2z', p.p, p.p'
+  float4 sh[28];                   // template cell: shift s h, entry code in .w
+  int end[28];                     // end of the template cell's candidates (flattened)
+  int off[28];                     // atom = candidate + off
+  uint8_t chunk[kTileCh][32];      // phase 2: chunk of an atom's w-th nonzero mask word
+};
+
 template <bool HALF>
-__global__ void __launch_bounds__(kBlk) k_build(Sys s, ListOut lo_) {
-  __shared__ uint32_t stage[2 * kGroup][kBlk];
+__global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, int slice_max) {
+  __shared__ BuildWarp sm_[kBWarps];
   if (!full_on(s) || s.half == 2) return;  // 2: forces straight from the cells, no list
+  BuildWarp &sm = sm_[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
   const int N = s.st->N;
   const size_t Nc = s.N_cap;
-  const float lo_thr = lo_.lo, hi_thr = lo_.hi;
-  const double rns2 = lo_.rns2;
+  const float mid = (float)lo_.rns2;
   const int ngroups = lo_.nmax / kGroup;
-  constexpr bool half = HALF;
-  const int tx = threadIdx.x;
-  for (int i = blockIdx.x * kBlk + tx; i < N; i += gridDim.x * kBlk) {
-    const float4 pi = __ldg(s.pf + i);
-    const Grid &g = s.grid[__float_as_uint(pi.w) >> 8];
-    const uint32_t cc = s.cellc[i];
-    const int c0 = cell_coord(cc, 0), c1 = cell_coord(cc, 1), c2 = cell_coord(cc, 2);
-    int count = 0;
-    auto flush = [&](int grp, int fill) {
-      if (grp >= ngroups) return;
-      const int h = (grp & 1) * kGroup;
-      const uint32_t pad = pad_entry(Nc);
-      uint32_t w[kGroup];
-#pragma unroll
-      for (int q = 0; q < kGroup; ++q) w[q] = q < fill ? stage[h + q][tx] : pad;
-      uint4 *o = reinterpret_cast<uint4 *>(lo_.nbr) + ((size_t)grp * Nc + i) * 2;
-      // lists are written once per build and read by the next pass from
-      // HBM: evict-first stores keep L2 for the records the builds gather
-      __stcs(o, make_uint4(w[0], w[1], w[2], w[3]));
-      __stcs(o + 1, make_uint4(w[4], w[5], w[6], w[7]));
-    };
-    for (int t = 0; t < 27; ++t) {
-      const int sx = t % 3 - 1, sy = (t / 3) % 3 - 1, sz = t / 9 - 1;
-      int cx, cy, cz, nx, ny, nz;
-      if (!stencil_cell(c0, sx, g.nc[0], g.per[0], &cx, &nx) ||
-          !stencil_cell(c1, sy, g.nc[1], g.per[1], &cy, &ny) ||
-          !stencil_cell(c2, sz, g.nc[2], g.per[2], &cz, &nz))
-        continue;
-      const int cj = dbg_idx(s, g.cell_off + cx + g.nc[0] * (cy + g.nc[1] * cz), s.n_cells);
-      const int a = s.cell_start[cj], b = dbg_idx(s, s.cell_start[cj + 1], s.N_cap + 1, a);
-      // d = p_j - q with q = p_i - s h (the shifted own offset, once per cell)
-      const float qx = pi.x - (float)sx * g.hf[0];
-      const float qy = pi.y - (float)sy * g.hf[1];
-      const float qz = pi.z - (float)sz * g.hf[2];
-      const int self = (nx == 0 && ny == 0 && nz == 0) ? i : -1;
-      const uint32_t code = pack_nbr(0, sx, sy, sz);
-      // half lists: an image of i itself is kept for the lexicographically
-      // positive stencil offset only (its mirror has the negative one)
-      const bool s_pos = sz > 0 || (sz == 0 && (sy > 0 || (sy == 0 && sx > 0)));
-      // blocks of four candidates; FULL: all four inside the cell's range
-      const float2 mqx = make_float2(-qx, -qx), mqy = make_float2(-qy, -qy),
-                   mqz = make_float2(-qz, -qz);
-      auto block4 = [&](const int j0, auto full) {
-        constexpr bool FULL = decltype(full)::value;
-        const int before = count;
-        float4 pj[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) pj[u] = __ldg(s.pf + (FULL ? j0 + u : min(j0 + u, b - 1)));
-        // r^2 of two candidates per packed FP32 instruction
-        float r2v[4];
-#pragma unroll
-        for (int pr = 0; pr < 2; ++pr) {
-          const float4 &qa = pj[2 * pr], &qb = pj[2 * pr + 1];
-          const float2 dx = __fadd2_rn(make_float2(qa.x, qb.x), mqx);
-          const float2 dy = __fadd2_rn(make_float2(qa.y, qb.y), mqy);
-          const float2 dz = __fadd2_rn(make_float2(qa.z, qb.z), mqz);
-          const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-          r2v[2 * pr] = r2.x;
-          r2v[2 * pr + 1] = r2.y;
+  const unsigned full = 0xffffffffu;
+  const int warps = gridDim.x * kBWarps;
+  for (int base = slice_max * (blockIdx.x * kBWarps + (threadIdx.x >> 5)); base < N;
+       base += slice_max * warps) {
+    // slices: every cell's atoms in equal parts of at most slice_max; this
+    // warp takes those that start in its slice_max atoms
+    int n_sl = 0;
+    bool lead = false;
+    if (lane < slice_max && base + lane < N) {
+      const uint32_t cc = s.cellc[base + lane];
+      const Grid &g = s.grid[s.info[base + lane] >> 8];
+      const int cell = dbg_idx(s, g.cell_off + cell_coord(cc, 0) +
+                                      g.nc[0] * (cell_coord(cc, 1) + g.nc[1] * cell_coord(cc, 2)),
+                               s.n_cells);
+      const int c0 = s.cell_start[cell], n = s.cell_start[cell + 1] - c0;
+      const int parts = (n + slice_max - 1) / slice_max;
+      const int sz = parts > 0 ? (n + parts - 1) / parts : 1;
+      const int k = base + lane - c0;
+      lead = k % sz == 0;
+      n_sl = min(sz, n - k);
+    }
+    for (unsigned leads = __ballot_sync(full, lead); leads; leads &= leads - 1) {
+      const int l0 = __ffs(leads) - 1;
+      const int a0 = base + l0, n = __shfl_sync(full, n_sl, l0);
+      const uint32_t cc = s.cellc[a0];
+      const Grid &g = s.grid[s.info[a0] >> 8];
+      const int c0 = cell_coord(cc, 0), c1 = cell_coord(cc, 1), c2 = cell_coord(cc, 2);
+      // ---- the candidates: 27 runs of atoms, flattened --------------------
+      int len = 0, first = 0;
+      float4 sh = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (lane < 27) {
+        const int sx = lane % 3 - 1, sy = (lane / 3) % 3 - 1, sz = lane / 9 - 1;
+        int cx, cy, cz, nx, ny, nz;
+        if (stencil_cell(c0, sx, g.nc[0], g.per[0], &cx, &nx) &&
+            stencil_cell(c1, sy, g.nc[1], g.per[1], &cy, &ny) &&
+            stencil_cell(c2, sz, g.nc[2], g.per[2], &cz, &nz)) {
+          const int cj = dbg_idx(s, g.cell_off + cx + g.nc[0] * (cy + g.nc[1] * cz), s.n_cells);
+          first = s.cell_start[cj];
+          len = dbg_idx(s, s.cell_start[cj + 1], s.N_cap + 1, first) - first;
         }
-        bool band = false;
+        sh = make_float4((float)sx * g.hf[0], (float)sy * g.hf[1], (float)sz * g.hf[2],
+                         __uint_as_float(pack_nbr(0, sx, sy, sz)));
+      }
+      int incl = len;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int j = j0 + u;
-          const float r2f = r2v[u];
-          const bool ok = (FULL || j < b) && j != self && (!half || half_keep(i, j, s_pos));
-          const bool acc = ok && r2f < lo_thr;
-          band = band || (ok && !acc && !(r2f > hi_thr));
-          stage[count & 15][tx] = code | ((uint32_t)j << 6);  // kept only if accepted
-          count += acc ? 1 : 0;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(full, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const int total = __shfl_sync(full, incl, 31);
+      // this lane's atom among the flattened candidates (template cell 13 is its own)
+      const int own = a0 + lane - __shfl_sync(full, first - (incl - len), 13);
+      const float bx = 0.6f * g.hf[0], by = 0.6f * g.hf[1], bz = 0.6f * g.hf[2];
+      // in its cell (false for NaN too)
+      auto inside = [&](const float4 &p) {
+        return fabsf(p.x) <= bx && fabsf(p.y) <= by && fabsf(p.z) <= bz;
+      };
+      __syncwarp();  // the previous slice's reads are done
+      if (lane < 28) {
+        sm.sh[lane] = sh;
+        sm.end[lane] = incl;  // lane 27: the total
+        sm.off[lane] = first - (incl - len);
+      }
+      bool out_a = false, far_a = false;
+      {
+        float4 p = make_float4(0.f, 0.f, 0.f, 1e30f);  // no atom: far from everything
+        if (lane < n) {
+          p = __ldg(s.pf + a0 + lane);
+          out_a = !inside(p);
+          p.w = fmaf(p.z, p.z, fmaf(p.y, p.y, p.x * p.x));
+          far_a = !(p.w == p.w);
         }
-        if (band) {
-          // rare: redo this block of four with the exact test where needed
-          count = before;
+        float *q = reinterpret_cast<float *>(&sm.a0[lane >> 1]) + (lane & 1);
+        q[0] = -2.f * p.x;
+        q[2] = -2.f * p.y;
+        q = reinterpret_cast<float *>(&sm.a1[lane >> 1]) + (lane & 1);
+        q[0] = -2.f * p.z;
+        q[2] = p.w;
+      }
+      __syncwarp();
+      int t = 0;      // this lane's template cell (moves up with its candidates)
+      int count = 0;  // this lane's atom
+      for (int tile = 0; tile < total; tile += 32 * kTileCh) {
+        const int n_ch = min(kTileCh, (total - tile + 31) >> 5);
+        // ---- phase 1: two chunks of 32 candidates at a time ---------------
+        float4 r2[2];  // the records of the next pair of chunks, loaded ahead
+        int j2[2], t2[2];
+        auto fetch = [&](int c) {
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int j = j0 + u;
-            const float r2f = r2v[u];
-            const bool ok = (FULL || j < b) && j != self && (!half || half_keep(i, j, s_pos));
-            bool acc = ok && r2f < lo_thr;
-            if (ok && !acc && !(r2f > hi_thr))
-              acc = exact_pair(s, g, i, code | ((uint32_t)j << 6), c0, c1, c2, rns2);
-            stage[count & 15][tx] = code | ((uint32_t)j << 6);
-            count += acc ? 1 : 0;
+          for (int h = 0; h < 2; ++h) {
+            const int p = tile + 32 * (c + h) + 31 - lane;
+            if (c < n_ch && p < total) {
+              while (p >= sm.end[t]) ++t;
+              t2[h] = t;
+              j2[h] = dbg_idx(s, p + sm.off[t], s.N_cap);
+              r2[h] = __ldg(s.pf + j2[h]);
+            } else {
+              t2[h] = -1;
+            }
+          }
+        };
+        fetch(0);
+        for (int c = 0; c < n_ch; c += 2) {
+          float4 q[2];  // shifted candidate, c.c - r_ns^2
+          uint32_t e[2];
+          bool out_c = out_a, far_c = far_a;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            q[h] = make_float4(0.f, 0.f, 0.f, 1e30f);
+            e[h] = 0;
+            if (t2[h] >= 0) {
+              const float4 r = r2[h], d = sm.sh[t2[h]];
+              e[h] = __float_as_uint(d.w) | ((uint32_t)j2[h] << 6);
+              const float x = r.x + d.x, y = r.y + d.y, z = r.z + d.z;
+              q[h] = make_float4(x, y, z, fmaf(z, z, fmaf(y, y, x * x)) - mid);
+              out_c = out_c || !inside(r);
+              far_c = far_c || !(r.x == r.x);
+            }
+            sm.ent[32 * (c + h) + lane] = e[h];
+          }
+          fetch(c + 2);
+          float near = 1e30f;  // smallest distance of a test from r_ns^2
+          auto keep = [&](int k, uint32_t ent) {
+            return !HALF || half_keep(a0 + k, nbr_j(ent), (ent & 63u) > 21u);
+          };
+#pragma unroll 2
+          for (int k = 0; k < n; k += 2) {
+            const float4 u = sm.a0[k >> 1], v = sm.a1[k >> 1];
+            unsigned b[4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              float2 d2 = __fadd2_rn(make_float2(q[h].w, q[h].w), make_float2(v.z, v.w));
+              d2 = __ffma2_rn(make_float2(q[h].x, q[h].x), make_float2(u.x, u.y), d2);
+              d2 = __ffma2_rn(make_float2(q[h].y, q[h].y), make_float2(u.z, u.w), d2);
+              d2 = __ffma2_rn(make_float2(q[h].z, q[h].z), make_float2(v.x, v.y), d2);
+              near = fminf(near, fminf(fabsf(d2.x), fabsf(d2.y)));
+              b[2 * h] = __ballot_sync(full, d2.x < 0.0f && keep(k, e[h]));
+              b[2 * h + 1] = __ballot_sync(full, d2.y < 0.0f && keep(k + 1, e[h]));
+            }
+            if (lane == 0) sm.mask[c >> 1][k >> 1] = make_uint4(b[0], b[1], b[2], b[3]);
+          }
+          const float width = __any_sync(full, out_c) ? 5.0f * s.build_band : s.build_band;
+          if (__any_sync(full, far_c || !(near > width))) {
+            // rare: the two chunks again, with the exact test where needed
+            __syncwarp();
+            for (int k = 0; k < n; ++k) {
+              const float *u = reinterpret_cast<const float *>(&sm.a0[k >> 1]) + (k & 1);
+              const float *v = reinterpret_cast<const float *>(&sm.a1[k >> 1]) + (k & 1);
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const float d2 = fmaf(q[h].z, v[0], fmaf(q[h].y, u[2], fmaf(q[h].x, u[0], q[h].w + v[2])));
+                bool acc = d2 < -width;
+                if (!acc && !(d2 > width) && tile + 32 * (c + h) + 31 - lane < total)
+                  acc = exact_pair(s, g, a0 + k, e[h], c0, c1, c2, lo_.rns2);
+                const unsigned b = __ballot_sync(full, acc && keep(k, e[h]));
+                if (lane == 0)
+                  reinterpret_cast<uint32_t *>(&sm.mask[c >> 1][k >> 1])[2 * h + (k & 1)] = b;
+              }
+            }
           }
         }
-        // a group of 8 completed in this block: write it out
-        if ((before >> 3) != (count >> 3)) flush(before >> 3, kGroup);
-      };
-      int j0 = a;
-      for (; j0 + 4 <= b; j0 += 4) block4(j0, std::true_type());
-      if (j0 < b) block4(j0, std::false_type());
-    }
-    if (count & 7) flush(count >> 3, count & 7);
-    lo_.nnbr[i] = count;
-    if (count > lo_.nmax) {
-      atomicOr(&s.st->bits, kStOverflow);
-      atomicMax(lo_.max_seen, count);
-      s.st->build_ovf = 1;
+        __syncwarp();
+        // an atom is no neighbour of itself (its images are)
+        uint32_t *mw = reinterpret_cast<uint32_t *>(sm.mask) + 4 * (lane >> 1) + (lane & 1);
+        auto word = [](int c) { return (c >> 1) * 64 + 2 * (c & 1); };
+        const int self = own - tile;
+        if (lane < n && (unsigned)self < (unsigned)(32 * n_ch))
+          mw[word(self >> 5)] &= ~(0x80000000u >> (self & 31));
+        // ---- phase 2: this lane's atom takes its accepted entries ----------
+        int words = 0, add = 0;  // its nonzero mask words (moved to the front), entries
+        for (int c = 0; c < n_ch; ++c) {
+          const uint32_t m = lane < n ? mw[word(c)] : 0u;
+          if (m) {
+            mw[word(words)] = m;
+            sm.chunk[words][lane] = (uint8_t)c;
+            ++words;
+          }
+          add += __popc(m);
+        }
+        uint32_t m = 0;
+        int at = 0;
+        const uint32_t *ent = sm.ent;
+        // the next accepted entry (the lane's list goes on with pad entries)
+        auto next = [&]() -> uint32_t {
+          if (m == 0 && at < words) {
+            m = mw[word(at)];
+            ent = sm.ent + 32 * sm.chunk[at][lane];
+            ++at;
+          }
+          const int b = 31 - __clz(m);
+          const uint32_t e = ent[max(b, 0)];
+          const bool some = m != 0;
+          m ^= some ? 1u << b : 0u;
+          return some ? e : pad_entry(Nc);
+        };
+        const int most = __reduce_max_sync(full, add);
+        if (tile == 0) {
+          for (int k = 0; k < most; k += kGroup) {
+            uint32_t w[kGroup];
+#pragma unroll
+            for (int q = 0; q < kGroup; ++q) w[q] = next();
+            if (k < add && (k >> 3) < ngroups) {
+              uint4 *o = reinterpret_cast<uint4 *>(lo_.nbr) + ((size_t)(k >> 3) * Nc + (a0 + lane)) * 2;
+              // lists are written once per build and read by the next pass from
+              // HBM: evict-first stores keep L2 for the records the builds gather
+              __stcs(o, make_uint4(w[0], w[1], w[2], w[3]));
+              __stcs(o + 1, make_uint4(w[4], w[5], w[6], w[7]));
+            }
+          }
+        } else {  // crowded cells: further tiles go on inside the last group
+          for (int k = 0; k < most; ++k) {
+            const uint32_t e = next();
+            if (k < add && ((count + k) >> 3) < ngroups) lo_.nbr[ell_index(count + k, a0 + lane, Nc)] = e;
+          }
+          if (lane < n)
+            for (int k = count + add; (k & 7) && (k >> 3) < ngroups; ++k)
+              lo_.nbr[ell_index(k, a0 + lane, Nc)] = pad_entry(Nc);
+        }
+        count += add;
+        __syncwarp();
+      }
+      if (lane < n) {
+        lo_.nnbr[a0 + lane] = count;
+        if (count > lo_.nmax) {
+          atomicOr(&s.st->bits, kStOverflow);
+          atomicMax(lo_.max_seen, count);
+          s.st->build_ovf = 1;
+        }
+      }
     }
   }
 }
@@ -893,13 +1068,15 @@ int launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_gra
   static int g_atom = 0, g_build = 0, g_cells = 0, g_filter = 0;
   if (g_atom == 0) {
     g_atom = persistent_blocks((const void *)k_bin, kBlk, 0);
-    g_build = persistent_blocks((const void *)k_build<false>, kBlk, 0);
+    // 4 rounds of blocks: slices differ, and the last round is a quarter of one
+    g_build = 4 * persistent_blocks((const void *)k_build<false>, 32 * kBWarps, 0);
     g_cells = persistent_blocks((const void *)k_cell_sort, kBlk, 0);
     g_filter = persistent_blocks((const void *)k_build_filter<false>, kBlk, 0);
   }
   const int gN = std::min(g_atom, nblk(s.N_cap > 0 ? s.N_cap : 1, kBlk));
   const int gC = std::min(g_cells, nblk(s.N_cap > 0 ? s.N_cap : 1, kBlk));
-  const int gB = std::min(g_build, nblk(s.N_cap > 0 ? s.N_cap : 1, kBlk));
+  const int slice = slice_atoms(s.N_cap);
+  const int gB = std::min(g_build, nblk(s.N_cap > 0 ? s.N_cap : 1, slice * kBWarps));
   const int gF = std::min(g_filter, nblk(s.N_cap > 0 ? s.N_cap : 1, kBlk));
   if (s.outer_on) {
     k_outer_disp<<<gN, kBlk, 0, st>>>(s);
@@ -923,14 +1100,14 @@ int launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_gra
   k_copyback<<<gN, kBlk, 0, st>>>(s);
   if (s.win_on) k_win_trim<<<1, 32, 0, st>>>(s);
   if (!s.outer_on) {
-    const ListOut lo{s.nbr, s.nnbr, s.nmax, s.rns2, s.filt_lo, s.filt_hi, &s.st->max_nnbr};
+    const ListOut lo{s.nbr, s.nnbr, s.nmax, s.rns2, &s.st->max_nnbr};
     if (s.half == 1)
-      k_build<true><<<gB, kBlk, 0, st>>>(s, lo);
+      k_build<true><<<gB, 32 * kBWarps, 0, st>>>(s, lo, slice);
     else
-      k_build<false><<<gB, kBlk, 0, st>>>(s, lo);
+      k_build<false><<<gB, 32 * kBWarps, 0, st>>>(s, lo, slice);
   } else {
-    const ListOut lo{s.nbr1, s.nnbr1, s.nmax1, s.rns2_1, s.filt1_lo, s.filt1_hi, &s.st->max_nnbr1};
-    k_build<false><<<gB, kBlk, 0, st>>>(s, lo);
+    const ListOut lo{s.nbr1, s.nnbr1, s.nmax1, s.rns2_1, &s.st->max_nnbr1};
+    k_build<false><<<gB, 32 * kBWarps, 0, st>>>(s, lo, slice);
     k_outer_refresh<<<gN, kBlk, 0, st>>>(s);
     if (s.half == 1)
       k_build_filter<true><<<gF, kBlk, 0, st>>>(s);

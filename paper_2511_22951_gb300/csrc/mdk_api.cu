@@ -373,8 +373,11 @@ void fill_sys_params(mdk_ctx *c) {
   {
     const double r1 = c->rc_list + (s.outer_on ? c->skin_outer : c->skin);
     s.rns2_1 = r1 * r1;
-    s.filt1_lo = (float)(s.rns2_1 * (1.0 - 1e-4));
-    s.filt1_hi = (float)(s.rns2_1 * (1.0 + 1e-4));
+    // k_build's FP32 test is off by less than 5e-6 h^2 (see there): 4 times that
+    double h = r1;
+    for (const Grid &g : c->grids)
+      for (int d = 0; d < 3; ++d) h = std::max(h, g.h[d]);
+    s.build_band = (float)(2e-5 * h * h);
     s.outer_budget = s.outer_on ? 0.5 * (c->skin_outer - c->skin) : 0.0;
   }
   s.half_skin2 = 0.25 * c->skin * c->skin;

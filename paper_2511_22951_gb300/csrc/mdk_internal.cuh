@@ -137,7 +137,9 @@ struct Sys {
   int red_chunks;           // chunks per replica (ceil of its largest atom count / kRedChunk)
   // list parameters
   double rns2;              // (rc + skin)^2
-  float filt_lo, filt_hi;   // FP32 pre-filter band around rns2
+  float filt_lo, filt_hi;   // FP32 pre-filter band around rns2 (filter builds)
+  float build_band;         // half width of the band around the squared radius of the list
+                            // that k_build makes from the cells (A^2)
   // outer list (two-level lists, outer_on != 0): every pair within
   // rc + skin_outer of the last full build, full kind; the Verlet list above is
   // filtered from it while every atom has moved less than outer_budget =
@@ -148,7 +150,6 @@ struct Sys {
   int32_t *nnbr1;
   uint32_t *nbr1;
   double rns2_1;            // (rc + skin_outer)^2
-  float filt1_lo, filt1_hi;
   double outer_budget;
   double half_skin2;        // (skin/2)^2
   int rebuild_every;
