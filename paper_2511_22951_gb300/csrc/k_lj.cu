@@ -184,12 +184,16 @@ __global__ void __launch_bounds__(256, lj_min_blocks<P, ENERGY, SHIFT>()) k_lj(S
     V pi;
     uint32_t inf = 0;
     R hx = 0, hy = 0, hz = 0;
+    Vec<P> geo;
     int nn = 0;
     if (valid) {
       pi = GP::ld(pg + i);
       inf = GP::info(pi);
       GP::h(s.grid[inf >> 8], hx, hy, hz);
-      h_scaled(hx, hy, hz);  // for s_scaled
+      if constexpr (sizeof(R) == 4)
+        h_scaled(hx, hy, hz);  // for s_scaled
+      else
+        geo = Vec<P>(pi, hx, hy, hz);
       nn = min(s.nnbr[i], s.nmax);
     }
     Acc<R> fx, fy, fz;
@@ -214,11 +218,10 @@ __global__ void __launch_bounds__(256, lj_min_blocks<P, ENERGY, SHIFT>()) k_lj(S
     walk<T>(
         s.nbr, Nc, i, nn, tl.t, [&](uint32_t j) { return GP::ld(pg + dbg_idx(s, j, Nc)); },
         [&](uint32_t ent, const V &pj) {
-          const R dx = pvec((R)pj.x, (R)pi.x, s_scaled(R(0), ent, 0), hx);
-          const R dy = pvec((R)pj.y, (R)pi.y, s_scaled(R(0), ent, 1), hy);
-          const R dz = pvec((R)pj.z, (R)pi.z, s_scaled(R(0), ent, 2), hz);
+          R dx, dy, dz;
+          geo.to(ent, pj, dx, dy, dz);
           const R r2 = r2_of(dx, dy, dz);
-          if (r2 < lc.rc2) {
+          if (below(r2, lc.rc2)) {
             R fr, v;
             lj_pair<GP, SHIFT, ENERGY>(lc, r2, fr, v);
             bx += fr * dx;

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(256, 4) k_lj_cells(Sys s, LJParams lp, StepArg
           const V pj = tl[k];
           const R dx = (R)pj.x - qx, dy = (R)pj.y - qy, dz = (R)pj.z - qz;
           const R r2 = dx * dx + dy * dy + dz * dz;
-          if (valid && r2 < lc.rc2 && j0 + k != self) {
+          if (valid && below(r2, lc.rc2) && j0 + k != self) {
             R fr, v;
             lj_pair<GP, SHIFT, ENERGY>(lc, r2, fr, v);
             fx.add(fr * dx);

@@ -28,6 +28,37 @@ __device__ __forceinline__ R herm_der(R t, R y0, R m0, R y1, R m1) {
   return d00 * (y0 - y1) + d10 * m0 + d11 * m1;
 }
 
+// ---- FP64 reciprocal and square roots of the pair loops -----------------------
+// GB300's FP64 pipe runs 2 lanes per clock and SM (1.26 TFLOP/s measured), so
+// it binds every FP64 pair loop and each operation counts: one FP64 warp
+// instruction takes the time of up to 64 others.  Both functions start from
+// the hardware approximation (about 20 bits) and take one step of the series
+// in its residual e: 1/x = y / (1 - e), e = 1 - x y, and 1/sqrt(x) =
+// y (1 - e)^(-1/2), e = 1 - x y^2, cut after e^2 (the rest is below 2^-58).
+// Valid for normal positive x; within 1 ulp (sqrt64: 1 ulp), 3 and 5
+// operations.
+__device__ __forceinline__ double rcp64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+// 1/sqrt(x) and sqrt(x)
+__device__ __forceinline__ void rsqrt64(double x, double &inv, double &root) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double t = x * y;
+  const double e = fma(-t, y, 1.0);
+  const double q = e * fma(e, 0.375, 0.5);
+  inv = fma(y, q, y);
+  root = fma(t, q, t);
+}
+// a < b for a >= 0 (or NaN: false), on the integer pipe
+__device__ __forceinline__ bool below(double a, double b) {
+  return (unsigned long long)__double_as_longlong(a) < (unsigned long long)__double_as_longlong(b);
+}
+__device__ __forceinline__ bool below(float a, float b) { return a < b; }
+
 // ---- gather-copy access per precision ---------------------------------------
 template <class P>
 struct G;
@@ -60,9 +91,17 @@ struct G<Fp64> {
     hy = g.h[1];
     hz = g.h[2];
   }
-  static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
-  static __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
-  static __device__ __forceinline__ double sqr(double x) { return sqrt(x); }
+  static __device__ __forceinline__ double rcp(double x) { return rcp64(x); }
+  static __device__ __forceinline__ double rsq(double x) {
+    double i, r;
+    rsqrt64(x, i, r);
+    return i;
+  }
+  static __device__ __forceinline__ double sqr(double x) {
+    double i, r;
+    rsqrt64(x, i, r);
+    return __double_as_longlong(x) >> 52 ? r : 0.0;  // 0 (and below the normal range): 0
+  }
   // EAM tables: (y_k, h m_k) per knot
   using Tab1 = double2;
   using Tab2 = double2;
@@ -227,7 +266,8 @@ __device__ __forceinline__ double s_scaled(double, uint32_t e, int d) {
 // order that every list kernel (and the packed LJ walk) shares: the
 // difference, then the shift by one FMA; r^2 = fma(dz, dz, fma(dy, dy, dx dx)).
 // Seen from j the vector is exactly minus the one seen from i, so both atoms
-// of a pair get the same r^2, bit for bit, and the same cutoff decision.
+// of a pair get the same r^2, bit for bit, and the same cutoff decision (FP32;
+// the FP64 kernels take Vec<Fp64>).
 __device__ __forceinline__ float pvec(float pj, float pi, float sh, float h) {
   return __fmaf_rn(sh, h, __fsub_rn(pj, pi));
 }
@@ -240,6 +280,52 @@ __device__ __forceinline__ float r2_of(float dx, float dy, float dz) {
 __device__ __forceinline__ double r2_of(double dx, double dy, double dz) {
   return __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
 }
+
+// One coordinate of an atom seen from its stencil's three layers along a
+// dimension, p - s h for s = -1, 0, 1: the FP64 pair vector component is
+// p_j - at(code of s), one FP64 operation; the choice is made by integer
+// selects (see rcp64).  Against (p_j - p_i) + s h the rounding of p - s h takes
+// the place of the difference's.
+struct Shift3 {
+  double a, b, c;
+  Shift3() = default;
+  __device__ __forceinline__ Shift3(double p, double h) : a(p + h), b(p), c(p - h) {}
+  __device__ __forceinline__ double at(uint32_t code) const {
+    code &= 3u;
+    const double q = code == 0u ? a : b;
+    return code == 2u ? c : q;
+  }
+};
+
+// The pair vector d = (p_j - p_i) + s h of list entry ent, per precision.
+template <class P>
+struct Vec;
+template <>
+struct Vec<Mixed> {
+  float x, y, z, hx, hy, hz;
+  Vec() = default;
+  __device__ __forceinline__ Vec(const float4 &p, float hx_, float hy_, float hz_)
+      : x(p.x), y(p.y), z(p.z), hx(hx_), hy(0.25f * hy_), hz(0.0625f * hz_) {}  // for s_scaled
+  __device__ __forceinline__ void to(uint32_t ent, const float4 &q, float &dx, float &dy,
+                                     float &dz) const {
+    dx = pvec(q.x, x, s_scaled(0.0f, ent, 0), hx);
+    dy = pvec(q.y, y, s_scaled(0.0f, ent, 1), hy);
+    dz = pvec(q.z, z, s_scaled(0.0f, ent, 2), hz);
+  }
+};
+template <>
+struct Vec<Fp64> {
+  Shift3 x, y, z;
+  Vec() = default;
+  __device__ __forceinline__ Vec(const dvec4 &p, double hx, double hy, double hz)
+      : x(p.x, hx), y(p.y, hy), z(p.z, hz) {}
+  __device__ __forceinline__ void to(uint32_t ent, const dvec4 &q, double &dx, double &dy,
+                                     double &dz) const {
+    dx = q.x - x.at(ent);
+    dy = q.y - y.at(ent >> 2);
+    dz = q.z - z.at(ent >> 4);
+  }
+};
 
 // the cell size scaled for s_scaled: (h_x, h_y / 4, h_z / 16)
 template <class R>

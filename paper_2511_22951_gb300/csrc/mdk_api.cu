@@ -889,25 +889,7 @@ int mdk_set_potential_lj(mdk_ctx *c, double eps, double sigma, double rc, int sh
   if (check_ctx(c)) return MDK_ERR_BAD_ARG;
   if (!(eps > 0.0) || !(sigma > 0.0) || !(rc > 0.0) || shift_mode < 0 || shift_mode > 2)
     return MDK_ERR_BAD_ARG;
-  LJParams &p = c->lj;
-  const double sr = sigma / rc, s6 = sr * sr * sr * sr * sr * sr;
-  const double u_rc = 4.0 * eps * (s6 * s6 - s6);
-  const double du_rc = -24.0 * eps * (2.0 * s6 * s6 - s6) / rc;
-  p.eps4 = 4.0 * eps;
-  p.eps24 = 24.0 * eps;
-  p.sig2 = sigma * sigma;
-  p.rc = rc;
-  p.rc2 = rc * rc;
-  p.u_shift = shift_mode >= 1 ? u_rc : 0.0;
-  p.du_rc = shift_mode == 2 ? du_rc : 0.0;
-  p.eps4f = (float)p.eps4;
-  p.eps24f = (float)p.eps24;
-  p.sig2f = (float)p.sig2;
-  p.rc2f = (float)p.rc2;
-  p.rcf = (float)rc;
-  p.u_shiftf = (float)p.u_shift;
-  p.du_rcf = (float)p.du_rc;
-  p.shift_mode = shift_mode;
+  lj_fill(c->lj, eps, sigma, rc, shift_mode);
   c->pot = 1;
   if (!c->planned) plan(c, rc, 0.3, 0, 0);
   return MDK_OK;

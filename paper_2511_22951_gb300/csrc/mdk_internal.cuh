@@ -216,9 +216,38 @@ __device__ __forceinline__ double dkey_inv(long long k) {
 
 struct LJParams {
   double eps4, eps24, sig2, rc2, u_shift, du_rc, rc;
+  // FP64 pair terms in powers of 1/r^2: V'(r)/r = r^-8 (f12 r^-6 + f6),
+  // V(r) = r^-6 (e12 r^-6 - e6) - shift
+  double f12, f6, e12, e6;
   float eps4f, eps24f, sig2f, rc2f, u_shiftf, du_rcf, rcf;
   int shift_mode;
 };
+
+inline void lj_fill(LJParams &p, double eps, double sigma, double rc, int shift_mode) {
+  const double sr = sigma / rc, s6 = sr * sr * sr * sr * sr * sr;
+  const double u_rc = 4.0 * eps * (s6 * s6 - s6);
+  const double du_rc = -24.0 * eps * (2.0 * s6 * s6 - s6) / rc;
+  p.eps4 = 4.0 * eps;
+  p.eps24 = 24.0 * eps;
+  p.sig2 = sigma * sigma;
+  p.rc = rc;
+  p.rc2 = rc * rc;
+  p.u_shift = shift_mode >= 1 ? u_rc : 0.0;
+  p.du_rc = shift_mode == 2 ? du_rc : 0.0;
+  p.eps4f = (float)p.eps4;
+  p.eps24f = (float)p.eps24;
+  p.sig2f = (float)p.sig2;
+  p.rc2f = (float)p.rc2;
+  p.rcf = (float)rc;
+  p.u_shiftf = (float)p.u_shift;
+  p.du_rcf = (float)p.du_rc;
+  p.shift_mode = shift_mode;
+  const long double q3 = (long double)sigma * sigma * sigma, q6 = q3 * q3, q12 = q6 * q6;
+  p.f12 = (double)(-48.0L * eps * q12);
+  p.f6 = (double)(24.0L * eps * q6);
+  p.e12 = (double)(4.0L * eps * q12);
+  p.e6 = (double)(4.0L * eps * q6);
+}
 
 // 32-byte FP64 gather-copy element (x, y, z, info bits in w)
 struct alignas(32) dvec4 {
