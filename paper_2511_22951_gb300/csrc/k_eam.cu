@@ -8,23 +8,16 @@
 // Pass 1 sums rho_i and evaluates F(rho_i), F'(rho_i) (FP64, once per atom);
 // pass 2 needs F'(rho_j) of every neighbour, so it is a second launch.  Both
 // run on a persistent grid; T lanes own one atom (autotuned), as in the LJ
-// kernel.  Where the spline tables are read from:
-//  * FP64: staged in shared memory once per block (160 KB for the force pass:
-//    one block per SM, up to 128 registers, no spills of the FP64 pair values);
-//  * mixed: straight from the workspace through L1 (80 KB per pass, which L1
-//    holds once no shared memory is carved out).  A pair's table load lands at
-//    a random knot; in shared memory the lanes of a quarter-warp then collide
-//    in banks (9.6 / 7.4 wavefronts per 16-byte load instead of 4), and an A/B
-//    on one GB300 measured L1 faster: cold-curve batch 1.18e9 against 1.07e9
-//    atom-timesteps/s, Al bulk and slab +1%.
+// kernel.  The spline tables are read from the workspace through L1, not
+// staged in shared memory.  Mixed (80 and 160 KB): a pair's load lands at a
+// random knot, where lanes collide in shared-memory banks (9.6 / 7.4
+// wavefronts per 16-byte load instead of 4), and an A/B on one GB300 measured
+// L1 faster: cold-curve batch 1.18e9 against 1.07e9 atom-timesteps/s, Al bulk
+// and slab +1%.  FP64 (160 and 320 KB of polynomial coefficients): the FP64
+// pipe binds, so the coefficients that save operations are worth their bytes.
 #include "k_pair.cuh"
 
 namespace mdk {
-
-// shared memory of the full-list passes (the mixed tables are read through L1)
-static int full_pass_smem(const EAMParams &p, int precision, int pass) {
-  return precision == 0 ? eam_smem_bytes(p, precision, pass) : 0;
-}
 
 namespace {
 
@@ -45,18 +38,7 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P>()) k_rho(Sys s, EAMPara
   using R = typename GP::R;
   using V = typename GP::V;
   using T1 = typename GP::Tab1;
-  extern __shared__ __align__(16) unsigned char smem[];
-  const T1 *rt;
-  if constexpr (sizeof(R) == 4) {
-    rt = GP::tab1(ep);  // mixed: through L1
-  } else {
-    T1 *w = reinterpret_cast<T1 *>(smem);
-    const T1 *src = GP::tab1(ep);
-    const int n = GP::n1(ep);
-    for (int q = threadIdx.x; q < n; q += blockDim.x) w[q] = src[q];
-    __syncthreads();
-    rt = w;
-  }
+  const T1 *rt = GP::tab1(ep);
   const int N = run_n(s.st);
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
@@ -68,12 +50,13 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P>()) k_rho(Sys s, EAMPara
     const int i = tl.atom(w);
     const bool valid = i < N;
     V pi;
-    R hx = 0, hy = 0, hz = 0;
+    Vec<P> geo;
     int nn = 0;
     if (valid) {
+      R hx, hy, hz;
       pi = GP::ld(pg + i);
       GP::h(s.grid[GP::info(pi) >> 8], hx, hy, hz);
-      h_scaled(hx, hy, hz);  // for s_scaled
+      geo = Vec<P>(pi, hx, hy, hz);
       nn = min(s.nnbr[i], s.nmax);
     }
     Acc<R> rho;
@@ -81,16 +64,13 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P>()) k_rho(Sys s, EAMPara
     walk<T>(
         s.nbr, Nc, i, nn, tl.t, [&](uint32_t j) { return GP::ld(pg + dbg_idx(s, j, Nc)); },
         [&](uint32_t ent, const V &pj) {
-          const R dx = pvec((R)pj.x, (R)pi.x, s_scaled(R(0), ent, 0), hx);
-          const R dy = pvec((R)pj.y, (R)pi.y, s_scaled(R(0), ent, 1), hy);
-          const R dz = pvec((R)pj.z, (R)pi.z, s_scaled(R(0), ent, 2), hz);
+          R dx, dy, dz;
+          geo.to(ent, pj, dx, dy, dz);
           const R r2 = r2_of(dx, dy, dz);
-          if (r2 < rc2) {
-            const R r = GP::sqr(r2);
-            const R u = r * inv_dr;
-            int kk = (int)u;
-            kk = kk > kmax ? kmax : kk;
-            const R t = u - (R)kk;
+          if (below(r2, rc2)) {
+            int kk;
+            R t;
+            GP::knot(r2, inv_dr, kmax, kk, t);
             br += GP::val1(rt, kk, t);
           }
         },
@@ -117,17 +97,11 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P, ENERGY>()) k_eam(Sys s,
   using R = typename GP::R;
   using V = typename GP::V;
   using TP = typename GP::TabPR;
-  extern __shared__ __align__(16) unsigned char smem[];
   const TP *tab;
-  if constexpr (sizeof(R) == 4) {
-    tab = GP::pr8(ep);  // mixed: through L1, one 32-byte record per interval
-  } else {
-    TP *w = reinterpret_cast<TP *>(smem);
-    const TP *src = GP::pr(ep);
-    for (int q = threadIdx.x; q < ep.nr; q += blockDim.x) w[q] = src[q];
-    __syncthreads();
-    tab = w;
-  }
+  if constexpr (sizeof(R) == 4)
+    tab = GP::pr8(ep);  // one 32-byte record per interval
+  else
+    tab = GP::pr(ep);
   const int N = run_n(s.st);
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
@@ -142,13 +116,15 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P, ENERGY>()) k_eam(Sys s,
     const bool valid = i < N;
     V pi;
     uint32_t inf = 0;
-    R hx = 0, hy = 0, hz = 0, fpi = 0;
+    R fpi = 0;
+    Vec<P> geo;
     int nn = 0;
     if (valid) {
+      R hx, hy, hz;
       pi = GP::ld(pg + i);
       inf = GP::info(pi);
       GP::h(s.grid[inf >> 8], hx, hy, hz);
-      h_scaled(hx, hy, hz);  // for s_scaled
+      geo = Vec<P>(pi, hx, hy, hz);
       fpi = __ldcs(fpa + i);
       nn = min(s.nnbr[i], s.nmax);
     }
@@ -162,18 +138,13 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P, ENERGY>()) k_eam(Sys s,
     walk<T>(
         s.nbr, Nc, i, nn, tl.t, [&](uint32_t j) { return GP::ld(pgf + dbg_idx(s, j, Nc)); },
         [&](uint32_t ent, const V &pj) {
-          const R dx = pvec((R)pj.x, (R)pi.x, s_scaled(R(0), ent, 0), hx);
-          const R dy = pvec((R)pj.y, (R)pi.y, s_scaled(R(0), ent, 1), hy);
-          const R dz = pvec((R)pj.z, (R)pi.z, s_scaled(R(0), ent, 2), hz);
+          R dx, dy, dz;
+          geo.to(ent, pj, dx, dy, dz);
           const R r2 = r2_of(dx, dy, dz);
-          if (r2 < rc2) {
-            const R inv_r = GP::rsq(r2);
-            const R r = r2 * inv_r;
-            const R u = r * inv_dr;
-            int kk = (int)u;
-            kk = kk > kmax ? kmax : kk;
-            const R t = u - (R)kk;
-            R dphi, drho, vphi = 0;
+          if (below(r2, rc2)) {
+            int kk;
+            R inv_r, t, dphi, drho, vphi = 0;
+            GP::knot(r2, inv_dr, kmax, inv_r, kk, t);
             if constexpr (sizeof(R) == 4) {
               float4 qa, qb;
               GP::ld_pr8(tab, kk, qa, qb);
@@ -183,7 +154,7 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P, ENERGY>()) k_eam(Sys s,
               GP::der_pr(tab, kk, t, dphi, drho);
               if (ENERGY) vphi = GP::val_pr(tab, ep, kk, t);
             }
-            const R fr = (dphi + (fpi + GP::fp_of(pj)) * drho) * inv_dr * inv_r;  // V'(r)/r
+            const R fr = GP::over_r(dphi, fpi + GP::fp_of(pj), drho, inv_dr, inv_r);  // V'(r)/r
             bx += fr * dx;
             by += fr * dy;
             bz += fr * dz;
@@ -251,7 +222,7 @@ __device__ __forceinline__ double hslope(const double *y, int n, int k) {
   return 0.5 * (y[k + 1] - y[k - 1]);
 }
 
-__global__ void k_eam_prepare(int nr, int nrho, const double *phi, const double *rho,
+__global__ void k_eam_prepare(int nr, int nrho, double rc, const double *phi, const double *rho,
                               const double *F, EAMTablesDev o) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < nr) {
@@ -268,12 +239,16 @@ __global__ void k_eam_prepare(int nr, int nrho, const double *phi, const double 
         k + 1 < nr ? make_float4((float)phi[k], (float)hslope(phi, nr, k + 1), 0.0f,
                                  (float)hslope(rho, nr, k + 1))
                    : make_float4((float)phi[k], 0.0f, 0.0f, 0.0f);
-    dvec4 q;
-    q.x = phi[k];
-    q.y = mp;
-    q.z = rho[k];
-    q.w = mr;
-    o.pr64[k] = q;
+    // cubics of the interval, y + t (m0 + t (3 D - 2 m0 - m1 + t (m0 + m1 - 2 D))), D = dy;
+    // their derivatives per unit of r
+    const double inv_dr = (double)(nr - 1) / rc;
+    const double mp1 = k + 1 < nr ? hslope(phi, nr, k + 1) : 0.0;
+    const double mr1 = k + 1 < nr ? hslope(rho, nr, k + 1) : 0.0;
+    const double p3 = (mp - dp) + (mp1 - dp), p2 = (dp - mp) - p3;
+    const double r3 = (mr - dr) + (mr1 - dr), r2 = (dr - mr) - r3;
+    o.rho_c64[k] = dvec4{rho[k], mr, r2, r3};
+    o.pr64[2 * k] = dvec4{mp * inv_dr, 2.0 * p2 * inv_dr, 3.0 * p3 * inv_dr, phi[k]};
+    o.pr64[2 * k + 1] = dvec4{mr * inv_dr, 2.0 * r2 * inv_dr, 3.0 * r3 * inv_dr, 0.0};
     if (k + 1 < nr)
       o.rho_i32[k] = make_float4((float)rho[k], (float)dr, (float)mr, (float)hslope(rho, nr, k + 1));
   }
@@ -306,19 +281,17 @@ int grid_for(K kern, int block, int smem, long long threads_needed) {
 
 template <class P, int MODE, bool EN, int T>
 void go(const Sys &s, const EAMParams &p, StepArgs a, int block, int prec, cudaStream_t st) {
-  const int b1 = full_pass_smem(p, prec, 1), b2 = full_pass_smem(p, prec, 2);
   auto k1 = k_rho<P, EN, T>;
   auto k2 = k_eam<P, MODE, EN, T>;
-  static int cb = 0, cs = -1, g1 = 0, g2 = 0, cap = -1;
-  if (cb != block || cs != b2 || cap != s.N_cap) {
-    g1 = grid_for(k1, block, b1, (long long)s.N_cap * T);
-    g2 = grid_for(k2, block, b2, (long long)s.N_cap * T);
+  static int cb = 0, g1 = 0, g2 = 0, cap = -1;
+  if (cb != block || cap != s.N_cap) {
+    g1 = grid_for(k1, block, 0, (long long)s.N_cap * T);
+    g2 = grid_for(k2, block, 0, (long long)s.N_cap * T);
     cb = block;
-    cs = b2;
     cap = s.N_cap;
   }
-  k1<<<g1, block, b1, st>>>(s, p, a);
-  k2<<<g2, block, b2, st>>>(s, p, a);
+  k1<<<g1, block, 0, st>>>(s, p, a);
+  k2<<<g2, block, 0, st>>>(s, p, a);
 }
 
 template <class P, int MODE, bool EN>
@@ -356,44 +329,13 @@ void by_mode(const Sys &s, const EAMParams &p, Mode m, StepArgs a, const LaunchC
     by_energy<P, kFinal>(s, p, a, c, prec, st);
 }
 
-template <class K>
-cudaError_t smem_attr(K k, int bytes) {
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-
-template <class P, int T>
-cudaError_t attrs_t(int b1, int b2) {
-  cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = smem_attr(k_rho<P, true, T>, b1);
-  if (e == cudaSuccess) e = smem_attr(k_rho<P, false, T>, b1);
-  if (e == cudaSuccess) e = smem_attr(k_eam<P, kForceOnly, true, T>, b2);
-  if (e == cudaSuccess) e = smem_attr(k_eam<P, kForceOnly, false, T>, b2);
-  if (e == cudaSuccess) e = smem_attr(k_eam<P, kStep, true, T>, b2);
-  if (e == cudaSuccess) e = smem_attr(k_eam<P, kStep, false, T>, b2);
-  if (e == cudaSuccess) e = smem_attr(k_eam<P, kFinal, true, T>, b2);
-  if (e == cudaSuccess) e = smem_attr(k_eam<P, kFinal, false, T>, b2);
-  return e;
-}
-
-template <class P>
-int attrs(int b1, int b2) {
-  cudaError_t e = attrs_t<P, 1>(b1, b2);
-  if (e == cudaSuccess) e = attrs_t<P, 2>(b1, b2);
-  if (e == cudaSuccess) e = attrs_t<P, 4>(b1, b2);
-  if (e == cudaSuccess) e = attrs_t<P, 8>(b1, b2);
-  if (e == cudaSuccess) e = attrs_t<P, 32>(b1, b2);
-  return e == cudaSuccess ? 0 : -1;
-}
-
 }  // namespace
 
+// tables that the mixed half-list passes stage in shared memory (the FP64
+// ones read theirs through L1)
 int eam_smem_bytes(const EAMParams &p, int precision, int pass) {
-  if (precision == 0) return p.nr * (int)(pass == 1 ? sizeof(double2) : sizeof(dvec4));
+  if (precision == 0) return 0;
   return pass == 1 ? (p.nr - 1) * (int)sizeof(float4) : p.nr * (int)sizeof(float4);
-}
-
-int configure_eam_smem(int b1, int b2, int precision) {
-  return precision == 0 ? attrs<Fp64>(b1, b2) : attrs<Mixed>(b1, b2);
 }
 
 void launch_eam(const Sys &s, const EAMParams &p, int precision, Mode mode, StepArgs a,
@@ -408,9 +350,8 @@ namespace {
 template <class P, int T>
 void rho_only(const Sys &s, const EAMParams &p, StepArgs a, int block, int prec,
               cudaStream_t st) {
-  const int b1 = full_pass_smem(p, prec, 1);
   auto k1 = k_rho<P, false, T>;
-  k1<<<grid_for(k1, block, b1, (long long)s.N_cap * T), block, b1, st>>>(s, p, a);
+  k1<<<grid_for(k1, block, 0, (long long)s.N_cap * T), block, 0, st>>>(s, p, a);
 }
 template <class P>
 void rho_by_tpa(const Sys &s, const EAMParams &p, StepArgs a, const LaunchCfg &c, int prec,
@@ -439,7 +380,7 @@ void launch_eam_rho(const Sys &s, const EAMParams &p, int precision, StepArgs a,
 void launch_eam_prepare(const EAMParams &p, const double *phi, const double *rho,
                         const double *F, EAMTablesDev out, cudaStream_t st) {
   const int n = p.nr > p.nrho ? p.nr : p.nrho;
-  k_eam_prepare<<<nblk(n, 256), 256, 0, st>>>(p.nr, p.nrho, phi, rho, F, out);
+  k_eam_prepare<<<nblk(n, 256), 256, 0, st>>>(p.nr, p.nrho, p.rc, phi, rho, F, out);
 }
 
 }  // namespace mdk

@@ -14,8 +14,9 @@
 //   k_eam_half   the pair force added to i and subtracted from j (rows 0-2),
 //                half of phi and of the pair virial to each atom
 //   k_half_fin   (k_lj_half.cu) takes the totals and finishes the step.
-// The tables are staged in shared memory on a persistent grid as in the
-// full-list passes.  Mixed path: 64-bit fixed-point accumulators (order-
+// Persistent grid; the mixed tables are staged in shared memory, the FP64
+// polynomial coefficients come through L1 as in the full-list passes.  Mixed
+// path: 64-bit fixed-point accumulators (order-
 // independent, reproducible); FP64 path: FP64 reduction atomics.
 #include "k_pair.cuh"
 
@@ -35,13 +36,14 @@ __global__ void __launch_bounds__(256, 2) k_rho_half(Sys s, EAMParams ep, StepAr
   using T1 = typename GP::Tab1;
   using Q = typename H::Q;
   extern __shared__ __align__(16) unsigned char smem[];
-  T1 *rt = reinterpret_cast<T1 *>(smem);
-  {
-    const T1 *src = GP::tab1(ep);
+  const T1 *rt = GP::tab1(ep);
+  if constexpr (sizeof(R) == 4) {
+    T1 *w = reinterpret_cast<T1 *>(smem);
     const int n = GP::n1(ep);
-    for (int q = threadIdx.x; q < n; q += blockDim.x) rt[q] = src[q];
+    for (int q = threadIdx.x; q < n; q += blockDim.x) w[q] = rt[q];
+    rt = w;
+    __syncthreads();
   }
-  __syncthreads();
   const int N = run_n(s.st);
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
@@ -53,21 +55,20 @@ __global__ void __launch_bounds__(256, 2) k_rho_half(Sys s, EAMParams ep, StepAr
     const V pi = GP::ld(pg + i);
     R hx, hy, hz;
     GP::h(s.grid[GP::info(pi) >> 8], hx, hy, hz);
-    h_scaled(hx, hy, hz);  // for s_scaled
+    const Vec<P> geo(pi, hx, hy, hz);
     const int nn = min(s.nnbr[i], s.nmax);
     Q rho = 0;
     walk<1>(
         s.nbr, Nc, i, nn, 0, [&](uint32_t j) { return GP::ld(pg + dbg_idx(s, j, Nc)); },
         [&](uint32_t ent, const V &pj) {
-          const R dx = pvec((R)pj.x, (R)pi.x, s_scaled(R(0), ent, 0), hx);
-          const R dy = pvec((R)pj.y, (R)pi.y, s_scaled(R(0), ent, 1), hy);
-          const R dz = pvec((R)pj.z, (R)pi.z, s_scaled(R(0), ent, 2), hz);
+          R dx, dy, dz;
+          geo.to(ent, pj, dx, dy, dz);
           const R r2 = r2_of(dx, dy, dz);
-          if (r2 < rc2) {
-            const R u = GP::sqr(r2) * inv_dr;
-            int kk = (int)u;
-            kk = kk > kmax ? kmax : kk;
-            const Q q = H::q(GP::val1(rt, kk, u - (R)kk));
+          if (below(r2, rc2)) {
+            int kk;
+            R t;
+            GP::knot(r2, inv_dr, kmax, kk, t);
+            const Q q = H::q(GP::val1(rt, kk, t));
             rho += q;
             H::red(acc + dbg_idx(s, nbr_j(ent), Nc, i), q);
           }
@@ -106,12 +107,13 @@ __global__ void __launch_bounds__(256, 2) k_eam_half(Sys s, EAMParams ep, StepAr
   using TP = typename GP::TabPR;
   using Q = typename H::Q;
   extern __shared__ __align__(16) unsigned char smem[];
-  TP *tab = reinterpret_cast<TP *>(smem);
-  {
-    const TP *src = GP::pr(ep);
-    for (int q = threadIdx.x; q < ep.nr; q += blockDim.x) tab[q] = src[q];
+  const TP *tab = GP::pr(ep);
+  if constexpr (sizeof(R) == 4) {
+    TP *w = reinterpret_cast<TP *>(smem);
+    for (int q = threadIdx.x; q < ep.nr; q += blockDim.x) w[q] = tab[q];
+    tab = w;
+    __syncthreads();
   }
-  __syncthreads();
   const int N = run_n(s.st);
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
@@ -128,26 +130,22 @@ __global__ void __launch_bounds__(256, 2) k_eam_half(Sys s, EAMParams ep, StepAr
     const V pi = GP::ld(pg + i);
     R hx, hy, hz;
     GP::h(s.grid[GP::info(pi) >> 8], hx, hy, hz);
-    h_scaled(hx, hy, hz);  // for s_scaled
+    const Vec<P> geo(pi, hx, hy, hz);
     const R fpi = fpa[i];
     const int nn = min(s.nnbr[i], s.nmax);
     Q fx = 0, fy = 0, fz = 0, e = 0, w0 = 0, w1 = 0, w2 = 0, w3 = 0, w4 = 0, w5 = 0;
     walk<1>(
         s.nbr, Nc, i, nn, 0, [&](uint32_t j) { return GP::ld(pgf + dbg_idx(s, j, Nc)); },
         [&](uint32_t ent, const V &pj) {
-          const R dx = pvec((R)pj.x, (R)pi.x, s_scaled(R(0), ent, 0), hx);
-          const R dy = pvec((R)pj.y, (R)pi.y, s_scaled(R(0), ent, 1), hy);
-          const R dz = pvec((R)pj.z, (R)pi.z, s_scaled(R(0), ent, 2), hz);
+          R dx, dy, dz;
+          geo.to(ent, pj, dx, dy, dz);
           const R r2 = r2_of(dx, dy, dz);
-          if (r2 < rc2) {
-            const R inv_r = GP::rsq(r2);
-            const R u = r2 * inv_r * inv_dr;
-            int kk = (int)u;
-            kk = kk > kmax ? kmax : kk;
-            const R t = u - (R)kk;
-            R dphi, drho;
+          if (below(r2, rc2)) {
+            int kk;
+            R inv_r, t, dphi, drho;
+            GP::knot(r2, inv_dr, kmax, inv_r, kk, t);
             GP::der_pr(tab, kk, t, dphi, drho);
-            const R fr = (dphi + (fpi + GP::fp_of(pj)) * drho) * inv_dr * inv_r;  // V'(r)/r
+            const R fr = GP::over_r(dphi, fpi + GP::fp_of(pj), drho, inv_dr, inv_r);  // V'(r)/r
             if (sizeof(R) == 4) bad = bad || !(fabs(fr) < fr_max);
             const Q qx = H::q(fr * dx), qy = H::q(fr * dy), qz = H::q(fr * dz);
             const size_t j = dbg_idx(s, nbr_j(ent), Nc, i);

@@ -102,34 +102,66 @@ struct G<Fp64> {
     rsqrt64(x, i, r);
     return __double_as_longlong(x) >> 52 ? r : 0.0;  // 0 (and below the normal range): 0
   }
-  // EAM tables: (y_k, h m_k) per knot
-  using Tab1 = double2;
+  // Interval and place in it of sqrt(r2): 1/sqrt(r2), k and t.  The floor is
+  // taken by one FMA rounded down at 2^52, whose low word is the integer, and
+  // t by one FMA (conversions run on the FP64 pipe): 3 operations after the
+  // root.  k is clamped on both sides: coinciding atoms give NaN.
+  static __device__ __forceinline__ void knot_at(double r, double inv_dr, int kmax, int &k,
+                                                 double &t) {
+    const double m = __fma_rd(r, inv_dr, 4503599627370496.0);
+    k = max(0, min((int)(unsigned)__double_as_longlong(m), kmax));
+    t = fma(r, inv_dr, 4503599627370496.0 - __hiloint2double(0x43300000, k));
+  }
+  static __device__ __forceinline__ void knot(double r2, double inv_dr, int kmax, double &inv_r,
+                                              int &k, double &t) {
+    double r;
+    rsqrt64(r2, inv_r, r);
+    knot_at(r, inv_dr, kmax, k, t);
+  }
+  static __device__ __forceinline__ void knot(double r2, double inv_dr, int kmax, int &k,
+                                              double &t) {
+    knot_at(sqr(r2), inv_dr, kmax, k, t);
+  }
+  // a 32-byte record of a polynomial table, through L1
+  static __device__ __forceinline__ dvec4 ld_rec(const dvec4 *p) {
+    dvec4 r;
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+        : "=d"(r.x), "=d"(r.y), "=d"(r.z), "=d"(r.w)
+        : "l"(p));
+    return r;
+  }
+  // EAM tables: the density's cubics; (y_k, h m_k) per knot for the adjoint
+  using Tab1 = dvec4;
   using Tab2 = double2;
-  static __device__ __forceinline__ const double2 *tab1(const EAMParams &e) { return e.rho64; }
+  static __device__ __forceinline__ const dvec4 *tab1(const EAMParams &e) { return e.rho_c64; }
   static __device__ __forceinline__ const double2 *rho2(const EAMParams &e) { return e.rho64; }
-  static __device__ __forceinline__ int n1(const EAMParams &e) { return e.nr; }
-  static __device__ __forceinline__ double val1(const double2 *t, int k, double u) {
-    const double2 a = t[k], b = t[k + 1];
-    return herm_val<double>(u, a.x, a.y, b.x, b.y);
+  static __device__ __forceinline__ double val1(const dvec4 *t, int k, double u) {
+    const dvec4 c = ld_rec(t + k);
+    return fma(fma(fma(c.w, u, c.z), u, c.y), u, c.x);
   }
   // h * derivative
   static __device__ __forceinline__ double der2(const double2 *t, int k, double u) {
     const double2 a = t[k], b = t[k + 1];
     return herm_der<double>(u, a.x, a.y, b.x, b.y);
   }
-  // force pass: interleaved phi / rho knots, h * derivatives of both
+  // force pass: derivatives with respect to r of both functions (and phi)
   using TabPR = dvec4;
   static __device__ __forceinline__ const dvec4 *pr(const EAMParams &e) { return e.pr64; }
   static __device__ __forceinline__ void der_pr(const dvec4 *t, int k, double u, double &dphi,
                                                 double &drho) {
-    const dvec4 a = t[k], b = t[k + 1];
-    dphi = herm_der<double>(u, a.x, a.y, b.x, b.y);
-    drho = herm_der<double>(u, a.z, a.w, b.z, b.w);
+    const dvec4 a = ld_rec(t + 2 * (size_t)k), b = ld_rec(t + 2 * (size_t)k + 1);
+    dphi = fma(fma(a.z, u, a.y), u, a.x);
+    drho = fma(fma(b.z, u, b.y), u, b.x);
   }
-  static __device__ __forceinline__ double val_pr(const dvec4 *t, const EAMParams &, int k,
+  static __device__ __forceinline__ double val_pr(const dvec4 *t, const EAMParams &e, int k,
                                                   double u) {
-    const dvec4 a = t[k], b = t[k + 1];
-    return herm_val<double>(u, a.x, a.y, b.x, b.y);
+    const dvec4 a = ld_rec(t + 2 * (size_t)k);
+    return fma(u * e.dr, fma(fma(a.z * (1.0 / 3.0), u, 0.5 * a.y), u, a.x), a.w);
+  }
+  // V'(r) / r from the derivatives of der_pr
+  static __device__ __forceinline__ double over_r(double dphi, double fsum, double drho, double,
+                                                  double inv_r) {
+    return fma(fsum, drho, dphi) * inv_r;
   }
   // gather copy with F'(rho) in place of the info word
   static __device__ __forceinline__ void st_fp(dvec4 *p, const dvec4 &q, double fp) {
@@ -160,6 +192,26 @@ struct G<Mixed> {
   static __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
   static __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
   static __device__ __forceinline__ float sqr(float x) { return sqrtf(x); }
+  static __device__ __forceinline__ void knot(float r2, float inv_dr, int kmax, float &inv_r,
+                                              int &k, float &t) {
+    inv_r = rsq(r2);
+    const float r = r2 * inv_r;
+    const float u = r * inv_dr;
+    k = (int)u;
+    k = k > kmax ? kmax : k;
+    t = u - (float)k;
+  }
+  static __device__ __forceinline__ void knot(float r2, float inv_dr, int kmax, int &k, float &t) {
+    const float r = sqr(r2);
+    const float u = r * inv_dr;
+    k = (int)u;
+    k = k > kmax ? kmax : k;
+    t = u - (float)k;
+  }
+  static __device__ __forceinline__ float over_r(float dphi, float fsum, float drho, float inv_dr,
+                                                 float inv_r) {
+    return (dphi + fsum * drho) * inv_dr * inv_r;
+  }
   // EAM tables rounded from FP64 differences (no FP32 cancellation):
   // density pass per interval (y_k, dy_k, h m_k, h m_{k+1}); rho per knot
   // (dy_k, h m_k) for the adjoint
@@ -167,7 +219,7 @@ struct G<Mixed> {
   using Tab2 = float2;
   static __device__ __forceinline__ const float4 *tab1(const EAMParams &e) { return e.rho_i32; }
   static __device__ __forceinline__ const float2 *rho2(const EAMParams &e) { return e.rho_d32; }
-  static __device__ __forceinline__ int n1(const EAMParams &e) { return e.nr - 1; }
+  static __device__ __forceinline__ int n1(const EAMParams &e) { return e.nr - 1; }  // staged
   static __device__ __forceinline__ float val1(const float4 *t, int k, float u) {
     const float4 q = t[k];
     const float u2 = u * u, u3 = u2 * u;

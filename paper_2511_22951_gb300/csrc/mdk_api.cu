@@ -240,7 +240,8 @@ size_t layout(mdk_ctx *c, char *base) {
   t.rho_d32 = cv.take<float2>(nr);
   t.phi_v32 = cv.take<float>(nr);
   t.pr32 = cv.take<float4>(nr);
-  t.pr64 = cv.take<dvec4>(nr);
+  t.rho_c64 = cv.take<dvec4>(nr);
+  t.pr64 = cv.take<dvec4>((size_t)2 * nr);
   t.pr8 = cv.take<float4>((size_t)2 * nr);
   c->adj_acc = cv.take<double2>((size_t)2 * nr + nrho);
   c->adj_out = cv.take<double>((size_t)2 * nr + nrho);
@@ -257,6 +258,7 @@ size_t layout(mdk_ctx *c, char *base) {
   c->eam.rho_d32 = t.rho_d32;
   c->eam.phi_v32 = t.phi_v32;
   c->eam.pr32 = t.pr32;
+  c->eam.rho_c64 = t.rho_c64;
   c->eam.pr64 = t.pr64;
   c->eam.pr8 = t.pr8;
   return align256(cv.off);
@@ -1159,9 +1161,7 @@ int mdk_set_workspace(mdk_ctx *c, void *dev_ptr, size_t bytes) {
                            cudaMemcpyHostToDevice, c->stream));
     launch_eam_prepare(e, kn, kn + e.nr, kn + 2 * e.nr, c->eam_dev, c->stream);
     MDK_CK(cudaPeekAtLastError());
-    if (configure_eam_smem(eam_smem_bytes(e, c->precision, 1), eam_smem_bytes(e, c->precision, 2),
-                           c->precision) ||
-        configure_eam_half_smem(eam_smem_bytes(e, c->precision, 1),
+    if (configure_eam_half_smem(eam_smem_bytes(e, c->precision, 1),
                                 eam_smem_bytes(e, c->precision, 2), c->precision))
       return MDK_ERR_CUDA;
   }

@@ -258,8 +258,13 @@ struct EAMParams {
   int nr, nrho;
   double rc, rc2, inv_dr, dr, rho_max, inv_drho, drho;
   float rc2f, inv_drf;
-  // FP64 knot tables (value, h * slope) per knot
+  // FP64 knot tables (value, h * slope) per knot (adjoint, embedding)
   const double2 *phi64, *rho64, *F64;
+  // FP64 polynomials per interval, t in [0, 1): density pass
+  //   rho_c64[k] = (c0, c1, c2, c3),  rho = c0 + t (c1 + t (c2 + t c3))
+  // force pass, derivatives with respect to r and the phi value
+  //   pr64[2k] = (b0, b1, b2, phi_k),  phi' = b0 + t (b1 + t b2);  pr64[2k + 1] the same of rho
+  const dvec4 *rho_c64, *pr64;
   // FP32 tables of the mixed path, rounded from FP64 quantities so that no
   // FP32 subtraction of neighbouring knot values is needed:
   //   rho_i32[k] = (y_k, y_{k+1} - y_k, h m_k, h m_{k+1})   (pass 1, rho value)
@@ -271,9 +276,7 @@ struct EAMParams {
   // force pass: phi and rho interleaved per knot, so one pair of loads
   // serves both derivatives
   //   pr32[k] = (phi_{k+1} - phi_k, h m^phi_k, rho_{k+1} - rho_k, h m^rho_k)
-  //   pr64[k] = (phi_k, h m^phi_k, rho_k, h m^rho_k)
   const float4 *pr32;
-  const dvec4 *pr64;
   // the full-list mixed force pass: one 32-byte record per interval k, read
   // with one 256-bit load per pair:
   //   pr8[2k] = pr32[k],  pr8[2k + 1] = (phi_k, h m^phi_{k+1}, 0, h m^rho_{k+1})
@@ -323,7 +326,7 @@ struct EAMTablesDev {
   float2 *rho_d32;
   float *phi_v32;
   float4 *pr32;
-  dvec4 *pr64;
+  dvec4 *rho_c64, *pr64;
   float4 *pr8;
 };
 
@@ -507,7 +510,6 @@ constexpr int kProfWidth = 24;
 void launch_profiles(const Sys &s, int axis, double origin, double bin_w, int nbins,
                      double cross_area, double *acc, cudaStream_t st);
 int eam_smem_bytes(const EAMParams &p, int precision, int pass);
-int configure_eam_smem(int bytes_pass1, int bytes_pass2, int precision);
 int configure_eam_half_smem(int bytes_pass1, int bytes_pass2, int precision);
 // half lists: density pass, embedding, force pass with accumulating atomics,
 // then launch_half_fin
