@@ -48,71 +48,96 @@ __global__ void __launch_bounds__(kBlk) k_kick_drift(Sys s, StepArgs a) {
     drift_publish<P>(s, a, i, inf, vx, vy, vz);
 }
 
-// ---- deterministic per-replica sums (fixed order, no atomics) -----------------------
-// Two passes: every block sums one chunk of kRedChunk atoms of one replica
-// (a fixed partition, so the result does not depend on the launch), then one
-// block per replica sums its chunks' partials in chunk order.  All SMs share
-// the first pass, so the sums of an 8.4M-atom system take a fraction of a
-// millisecond instead of one SM's tens of milliseconds.
+// ---- deterministic per-replica sums (fixed order, no atomics on the sums) -----------
+// Every block sums one chunk of atoms of one replica (a fixed partition, so
+// the result does not depend on the launch) and counts itself in; the block
+// that completes a replica adds its chunks' partials in chunk order and hands
+// the totals out.  The FP64 pipe of one SM binds a block, so chunks are small
+// (red_chunk_for) and the block sum of eight values takes 9 additions per lane
+// (block_sum8).  9,724 atoms 57 -> 9 us (two launches, 8192 atoms per block
+// and 40 additions per lane before, plus two device copies per replica where
+// the caller wants E and the virial), 8,388,608 atoms 168 -> 133 us.
 constexpr int kRedThreads = 256;
-constexpr int kRedTop = 1024;
 
-// the block's sums of acc[0..7] (fixed shuffle tree, then warps in order);
-// value c ends in thread c (c < 8)
-template <int NT>
+// The block's sums of acc[0..7]; thread c < 8 gets the sum of value c.  Three
+// exchanges halve the values that a lane carries while they double the lanes
+// that are summed (lane l ends with value (l >> 2) & 7 in bit-reversed order),
+// two more finish the warp; then warps in order.
 __device__ __forceinline__ double block_sum8(double (&acc)[8]) {
-  __shared__ double sh[8][NT / 32];
+  __shared__ double sh[8][kRedThreads / 32];
+  const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double v4[4], v2[2];
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    double v = acc[c];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[c][wid] = v;
+  for (int c = 0; c < 4; ++c) {
+    const bool up = lane & 16;
+    const double keep = up ? acc[c + 4] : acc[c], give = up ? acc[c] : acc[c + 4];
+    v4[c] = keep + __shfl_xor_sync(full, give, 16);
   }
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const bool up = lane & 8;
+    const double keep = up ? v4[c + 2] : v4[c], give = up ? v4[c] : v4[c + 2];
+    v2[c] = keep + __shfl_xor_sync(full, give, 8);
+  }
+  const bool up = lane & 4;
+  double v = (up ? v2[1] : v2[0]) + __shfl_xor_sync(full, up ? v2[0] : v2[1], 4);
+  v += __shfl_xor_sync(full, v, 2);
+  v += __shfl_xor_sync(full, v, 1);
+  if ((lane & 3) == 0) sh[lane >> 2][wid] = v;
   __syncthreads();
   double t = 0.0;
   if (threadIdx.x < 8)
-    for (int w = 0; w < NT / 32; ++w) t += sh[threadIdx.x][w];
+#pragma unroll
+    for (int w = 0; w < kRedThreads / 32; ++w) t += sh[threadIdx.x][w];
   return t;
 }
 
-__global__ void __launch_bounds__(kRedThreads) k_reduce_chunks(Sys s, int with_ke) {
-  const int r = blockIdx.x;
+__global__ void __launch_bounds__(kRedThreads) k_reduce(Sys s, int with_ke, double *E,
+                                                       double *virial) {
+  __shared__ bool last;
+  const int r = blockIdx.x, k = blockIdx.y;
   const Grid &g = s.grid[r];
   const int n = (s.n_rep == 1) ? s.st->N : g.n_atoms;
   const size_t Nc = s.N_cap;
-  for (int k = blockIdx.y; k < s.red_chunks; k += gridDim.y) {
-    const int q1 = min(n, (k + 1) * kRedChunk);
-    double acc[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) acc[c] = 0.0;
-    for (int q = k * kRedChunk + threadIdx.x; q < q1; q += kRedThreads) {
-      const int i = g.atom_off + q;
-      acc[0] += with_ke ? s.ka[i] : 0.0;
-      acc[1] += s.ea[i];
-#pragma unroll
-      for (int c = 0; c < 6; ++c) acc[2 + c] += s.wa[c * Nc + i];
-    }
-    const double t = block_sum8<kRedThreads>(acc);
-    if (threadIdx.x < 8) s.red_part[((size_t)r * s.red_chunks + k) * 8 + threadIdx.x] = t;
-    __syncthreads();  // block_sum8's shared slots are reused by the next chunk
-  }
-}
-
-__global__ void __launch_bounds__(kRedTop) k_reduce_top(Sys s) {
-  const int r = blockIdx.x;
+  const int q1 = min(n, (k + 1) * s.red_chunk);
   double acc[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) acc[c] = 0.0;
-  const double *p = s.red_part + (size_t)r * s.red_chunks * 8;
-  for (int k = threadIdx.x; k < s.red_chunks; k += kRedTop) {
+#pragma unroll 4
+  for (int q = k * s.red_chunk + threadIdx.x; q < q1; q += kRedThreads) {
+    const int i = g.atom_off + q;
+    if (with_ke) acc[0] += s.ka[i];
+    acc[1] += s.ea[i];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) acc[c] += p[(size_t)k * 8 + c];
+    for (int c = 0; c < 6; ++c) acc[2 + c] += s.wa[c * Nc + i];
   }
-  const double t = block_sum8<kRedTop>(acc);
-  if (threadIdx.x < 8) s.red[r * 9 + threadIdx.x] = t;
-  if (threadIdx.x == 0) s.red[r * 9 + 8] = (double)((s.n_rep == 1) ? s.st->N : s.grid[r].n_atoms);
+  double t = block_sum8(acc);
+  double *part = s.red_part + (size_t)r * s.red_chunks * 8;
+  if (threadIdx.x < 8) {
+    part[(size_t)k * 8 + threadIdx.x] = t;
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(s.red_done + r, 1u) == (unsigned)s.red_chunks - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+#pragma unroll
+  for (int c = 0; c < 8; ++c) acc[c] = 0.0;
+  for (int q = threadIdx.x; q < s.red_chunks; q += kRedThreads) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) acc[c] += __ldcg(part + (size_t)q * 8 + c);
+  }
+  t = block_sum8(acc);
+  const int c = threadIdx.x;
+  if (c < 8) s.red[r * 9 + c] = t;
+  if (E && c == 1) E[r] = t;
+  if (virial && c >= 2 && c < 8) virial[6 * r + c - 2] = t;
+  if (c == 0) {
+    s.red[r * 9 + 8] = (double)n;
+    s.red_done[r] = 0u;
+  }
 }
 
 // ---- state in / out in the caller's order -------------------------------------------
@@ -182,13 +207,10 @@ void launch_kick_drift(const Sys &s, int precision, StepArgs a, cudaStream_t st)
     k_kick_drift<Mixed><<<g, kBlk, 0, st>>>(s, a);
 }
 
-int launch_reduce(const Sys &s, int with_ke, cudaStream_t st) {
-  k_reduce_chunks<<<dim3(s.n_rep, std::min(s.red_chunks, 65535)), kRedThreads, 0, st>>>(s,
-                                                                                      with_ke);
-  k_reduce_top<<<s.n_rep, kRedTop, 0, st>>>(s);
-  return 2;
+int launch_reduce(const Sys &s, int with_ke, double *E, double *virial, cudaStream_t st) {
+  k_reduce<<<dim3(s.n_rep, s.red_chunks), kRedThreads, 0, st>>>(s, with_ke, E, virial);
+  return 1;
 }
-
 
 namespace {
 template <class P>

@@ -225,8 +225,10 @@ size_t layout(mdk_ctx *c, char *base) {
     int64_t per = c->n_rep == 1 ? (int64_t)Nc : 1;
     if (c->n_rep > 1)
       for (const Grid &g : c->grids) per = std::max<int64_t>(per, g.n_atoms);
-    s.red_chunks = (int)std::max<int64_t>(1, (per + kRedChunk - 1) / kRedChunk);
+    s.red_chunk = red_chunk_for(per);
+    s.red_chunks = (int)std::max<int64_t>(1, (per + s.red_chunk - 1) / s.red_chunk);
     s.red_part = cv.take<double>((size_t)8 * c->n_rep * s.red_chunks);
+    s.red_done = cv.take<unsigned>(c->n_rep);
   }
   c->thermo_ring = cv.take<double>((size_t)std::max(c->thermo_cap, 1) * c->n_rep * 10);
   // EAM tables: raw knots, (y, h m) FP64 and FP32 copies
@@ -1124,6 +1126,7 @@ int mdk_set_workspace(mdk_ctx *c, void *dev_ptr, size_t bytes) {
   fill_sys_params(c);
   Sys &s = c->sys;
   MDK_CK(cudaMemsetAsync(s.st, 0, sizeof(DevStatus), c->stream));
+  MDK_CK(cudaMemsetAsync(s.red_done, 0, sizeof(unsigned) * c->n_rep, c->stream));
   launch_init_far(s, c->precision, c->stream);
   MDK_CK(cudaMemsetAsync(s.cell_cnt, 0, sizeof(int32_t) * (c->n_cells + 1), c->stream));
   MDK_CK(cudaMemsetAsync(s.hacc, 0, sizeof(long long) * 10 * (size_t)std::max<int64_t>(c->N_cap, 1),
@@ -1565,7 +1568,7 @@ int mdk_compute(mdk_ctx *c, double *E, double *F, double *virial, int on_device)
   Sys &s = c->sys;
   r = force_pass(c, kForceOnly, 1, 0.0);
   if (r) return r;
-  c->launches += launch_reduce(s, 0, c->stream);
+  c->launches += launch_reduce(s, 0, on_device ? E : nullptr, on_device ? virial : nullptr, c->stream);
   MDK_CK(cudaPeekAtLastError());
   c->forces_valid = true;
   c->per_atom_valid = true;
@@ -1579,12 +1582,6 @@ int mdk_compute(mdk_ctx *c, double *E, double *F, double *virial, int on_device)
   }
   if (on_device) {
     if (F) launch_store_forces(s, F, c->stream);
-    for (int q = 0; q < R; ++q) {
-      if (E) MDK_CK(cudaMemcpyAsync(E + q, s.red + 9 * q + 1, sizeof(double),
-                                    cudaMemcpyDeviceToDevice, c->stream));
-      if (virial) MDK_CK(cudaMemcpyAsync(virial + 6 * q, s.red + 9 * q + 2, 6 * sizeof(double),
-                                         cudaMemcpyDeviceToDevice, c->stream));
-    }
     MDK_CK(cudaPeekAtLastError());
     return MDK_OK;
   }
@@ -1739,7 +1736,7 @@ int mdk_step(mdk_ctx *c, double dt, int64_t nsteps) {
     r = force_pass(c, last ? kFinal : kStep, thermo, dt);
     if (r) return r;
     if (thermo) {
-      c->launches += launch_reduce(s, 1, c->stream) + 1;
+      c->launches += launch_reduce(s, 1, nullptr, nullptr, c->stream) + 1;
       const int slot = (int)(c->thermo_written % std::max(c->thermo_cap, 1));
       k_thermo_store<<<1, std::max(32, ((c->n_rep + 31) / 32) * 32), 0, c->stream>>>(
           s, c->thermo_ring, slot, (double)gstep);

@@ -133,8 +133,10 @@ struct Sys {
   Grid *grid;
   DevStatus *st;
   double *red;              // reductions: per replica [K, U, W0..W5, N]
-  double *red_part;         // per replica and chunk of kRedChunk atoms: the 8 partial sums
-  int red_chunks;           // chunks per replica (ceil of its largest atom count / kRedChunk)
+  double *red_part;         // per replica and chunk of red_chunk atoms: the 8 partial sums
+  unsigned *red_done;       // per replica: chunks summed so far (0 between calls)
+  int red_chunk;            // atoms per chunk (red_chunk_for)
+  int red_chunks;           // chunks per replica (ceil of the largest atom count / red_chunk)
   // list parameters
   double rns2;              // (rc + skin)^2
   float filt_lo, filt_hi;   // FP32 pre-filter band around rns2 (filter builds)
@@ -344,8 +346,13 @@ __device__ __forceinline__ double cell_center(const Grid &g, int d, int c) {
 // entries with two 16-byte loads, a warp reads 1 KB contiguous, and the build
 // writes whole sectors (no partial-sector read-modify-write in L2).
 constexpr int kGroup = 8;
-// atoms per block of the first pass of the per-replica sums
-constexpr int kRedChunk = 8192;
+// Atoms per block of the per-replica sums, from the largest replica's atom
+// count: 1024 keeps one SM's FP64 pipe (2 lanes a clock) to ~2 us; at most 1024
+// chunks, so that the block that adds them up takes as long.
+inline int red_chunk_for(long long atoms) {
+  const long long k = (atoms + 1024LL * 1024 - 1) / (1024LL * 1024);
+  return 1024 * (int)(k > 1 ? k : 1);
+}
 __host__ __device__ __forceinline__ size_t ell_index(int k, int i, size_t Nc) {
   return ((size_t)(k >> 3) * Nc + (size_t)i) * kGroup + (size_t)(k & 7);
 }
@@ -492,8 +499,9 @@ void launch_lj_half(const Sys &s, const LJParams &p, int precision, Mode mode, S
 void launch_eam(const Sys &s, const EAMParams &p, int precision, Mode mode, StepArgs a,
                 const LaunchCfg &cfg, cudaStream_t st);
 void launch_kick_drift(const Sys &s, int precision, StepArgs a, cudaStream_t st);
-// returns the number of kernels launched
-int launch_reduce(const Sys &s, int with_ke, cudaStream_t st);
+// per-replica sums into s.red, and E [n_rep] / virial [n_rep][6] (device) unless
+// null; returns the number of kernels launched
+int launch_reduce(const Sys &s, int with_ke, double *E, double *virial, cudaStream_t st);
 void launch_eam_prepare(const EAMParams &p, const double *phi, const double *rho,
                         const double *F, EAMTablesDev out, cudaStream_t st);
 // the far records at index N_cap of both gather copies (see pad_entry)

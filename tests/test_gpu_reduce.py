@@ -76,3 +76,27 @@ def test_batched_replicas_one_or_several_chunks(mdk):
     ends = np.cumsum(sizes)
     check_totals(E, Wv, U, Wa, list(zip(np.r_[0, ends[:-1]], ends)))
     ctx.close()
+
+
+def test_device_outputs_equal_host_outputs(mdk):
+    """E and virial written by the sums' kernel itself (on_device), for a batch
+    and a single system, and with either output left out."""
+    import torch
+    rng = np.random.default_rng(7)
+    reps = [W.lattice_system(rng, (k, k, k), 5.26, W.MASS_AR, 0.0, sigma_jitter=0.05)
+            for k in (4, 5, 7)]
+    for rs in (reps, reps[2:]):
+        n = [r.n for r in rs]
+        ctx = mdk.Context([r.lo for r in rs], [r.hi for r in rs], [r.periodic for r in rs],
+                          np.concatenate([r.masses for r in rs]), "fp64", n_atoms=n)
+        ctx.set_potential_lj(W.LJ_AR.eps, W.LJ_AR.sigma, W.LJ_AR.rc, 1)
+        ctx.plan(W.LJ_AR.rc, 0.3)
+        ctx.set_state(np.concatenate([r.x for r in rs]))
+        E, F, Wv = ctx.compute()
+        Ed = torch.full((len(rs),), 7.0, dtype=torch.float64, device="cuda")
+        Wd = torch.full((len(rs), 6), 7.0, dtype=torch.float64, device="cuda")
+        ctx.compute_device(Ed, None, None)
+        ctx.compute_device(None, None, Wd)
+        torch.cuda.synchronize()
+        assert np.array_equal(Ed.cpu().numpy(), E) and np.array_equal(Wd.cpu().numpy(), Wv)
+        ctx.close()
