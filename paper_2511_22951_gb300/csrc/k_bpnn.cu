@@ -15,25 +15,37 @@
 //     pair vector u_a, R_a, f_c(R_a), f_c'(R_a) and exp(-eta_p R_a^2) for
 //     every (eta, kind) group p of the angular functions;
 //  2. radial functions, lanes over neighbours; angular functions, lanes over
-//     unordered pairs {a, b}; warp sums;
+//     unordered pairs {a, b}; warp sums.  G4 terms vanish for R_ab >= R_c (53%
+//     of the pairs of points in a sphere of radius R_c), so with G4 functions
+//     only every lane first queues its pairs inside R_c and then evaluates
+//     those, in their order (the zeros it leaves out change no sum);
 //  3. the network forward and reverse pass (lanes over hidden units, weights
 //     staged in shared memory per block) gives E_i and dE_i/dG;
 //  4. the gradients g_a = dE_i/dR_(j_a): every unordered pair {a, b} is
 //     evaluated once and gives, for its angular terms T(u_a, u_b, s = u_b -
 //     u_a), dT/du_a - dT/ds to a and dT/du_b + dT/ds to b.  The pairs run in
-//     a rotation schedule -- round k pairs a with (a + k) mod n -- so in one
-//     warp instruction no two lanes touch the same neighbour's shared sums
-//     (no atomics, and a fixed summation order: reproducible).  Per pair the
-//     angular functions are folded group by group: for each (eta, kind)
-//     group the sums over its functions of w A and w dA/dc (w = dE_i/dG)
-//     multiply the group's Gaussian-cutoff factor and its derivatives.
+//     a rotation schedule -- round k pairs a with (a + k) mod n, those inside
+//     R_c packed to the front -- so in one warp instruction no two lanes
+//     touch the same neighbour's shared sums (no atomics, and a fixed
+//     summation order: reproducible).  Per pair the angular functions are
+//     folded group by group: for each (eta, kind) group the sums over its
+//     functions of w A and w dA/dc (w = dE_i/dG) multiply the group's
+//     Gaussian-cutoff factor and its derivatives.
 //     Atom j_a receives -g_a, atom i receives sum_a g_a (E_i depends on
 //     relative positions only), and i keeps the virial -sum_a u_a (x) g_a of
 //     its own energy.  Forces are added to the per-atom
 // accumulators s.hacc (64-bit fixed point in the mixed path, FP64 atomics in
 // the FP64 path); launch_half_fin then finishes the step.  The mixed path
 // computes in FP32; a neighbour gradient at or above 2^22 eV/A sets the
-// non-finite status.
+// sets the non-finite status.
+//
+// FP32 issue binds: packed FP32 instructions (two lanes of a register pair)
+// carry the lambda = +-1 functions of a zeta group together, and in the
+// gradients two (eta, kind) groups.  131,072 atoms of the Al-like lattice (54
+// neighbours, 1431 pairs, 670 of them inside R_c): 5.40 ms a pass with every
+// pair and scalar FP32 (37,100 warp instructions per atom, issue 72%), 3.49 ms
+// now (19,500, issue 57%: 16 warps per SM, shared-memory latency and the
+// packed instructions' two cycles).
 #include "k_pair.cuh"
 
 namespace mdk {
@@ -68,110 +80,105 @@ struct BM<double> {
   static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
 };
 
+// two values side by side: one packed instruction in FP32, two in FP64
+template <class R>
+struct P2 {
+  R x, y;
+};
+template <class R>
+__device__ __forceinline__ P2<R> both(R v) {
+  return {v, v};
+}
+__device__ __forceinline__ P2<float> mul2(P2<float> a, P2<float> b) {
+  const float2 r = __fmul2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+  return {r.x, r.y};
+}
+__device__ __forceinline__ P2<float> fma2(P2<float> a, P2<float> b, P2<float> c) {
+  const float2 r =
+      __ffma2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y), make_float2(c.x, c.y));
+  return {r.x, r.y};
+}
+__device__ __forceinline__ P2<double> mul2(P2<double> a, P2<double> b) {
+  return {a.x * b.x, a.y * b.y};
+}
+__device__ __forceinline__ P2<double> fma2(P2<double> a, P2<double> b, P2<double> c) {
+  return {fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)};
+}
+
 // a parameter in the pair precision
 template <class R>
 __device__ __forceinline__ R pick(double d, float f) {
   return sizeof(R) == 8 ? (R)d : (R)f;
 }
 
-// x^e for a small non-negative integer e (uniform across the warp)
+// the per-slot weights of one (eta, kind) group, (lambda = +1, -1) per zeta
+// group, with vector loads
 template <class R>
-__device__ __forceinline__ R ipow(R x, int e) {
-  R r = R(1);
-  while (e) {
-    if (e & 1) r *= x;
-    x *= x;
-    e >>= 1;
-  }
-  return r;
-}
-
-// the 2 kBpZ per-slot weights of one (eta, kind) group, with vector loads
-template <class R>
-__device__ __forceinline__ void ld_group(const R *w, R out[2 * kBpZ]) {
-  if (sizeof(R) == 4) {
+__device__ __forceinline__ void ld_group(const R *w, P2<R> out[kBpZ]) {
+  if constexpr (sizeof(R) == 4) {
     const float4 *q = reinterpret_cast<const float4 *>(w);
 #pragma unroll
     for (int v = 0; v < kBpZ / 2; ++v) {
       const float4 a = q[v];
-      out[4 * v] = a.x;
-      out[4 * v + 1] = a.y;
-      out[4 * v + 2] = a.z;
-      out[4 * v + 3] = a.w;
+      out[2 * v].x = a.x;
+      out[2 * v].y = a.y;
+      out[2 * v + 1].x = a.z;
+      out[2 * v + 1].y = a.w;
     }
   } else {
     const double2 *q = reinterpret_cast<const double2 *>(w);
 #pragma unroll
     for (int v = 0; v < kBpZ; ++v) {
       const double2 a = q[v];
-      out[2 * v] = a.x;
-      out[2 * v + 1] = a.y;
+      out[v].x = a.x;
+      out[v].y = a.y;
     }
   }
 }
 
-// x^e and y^e together (one loop, uniform across the warp)
+// both components to a small non-negative integer power (uniform across the warp)
 template <class R>
-__device__ __forceinline__ void ipow2(R x, R y, int e, R &rx, R &ry) {
-  rx = R(1);
-  ry = R(1);
+__device__ __forceinline__ P2<R> ipow2(P2<R> x, int e) {
+  P2<R> r = both(R(1));
   while (e) {
-    if (e & 1) {
-      rx *= x;
-      ry *= y;
-    }
-    x *= x;
-    y *= y;
+    if (e & 1) r = mul2(r, x);
+    x = mul2(x, x);
     e >>= 1;
   }
+  return r;
 }
 
-// Powers of the angular term per zeta group: x = 1 + c, y = 1 - c.  ZS = 1
+// Powers of the angular term per zeta group: x = (1 + c, 1 - c).  ZS = 1
 // is the zeta set {1, 2, 4, 16} (zeta group z holds zeta = 1, 2, 4, 16): the
 // powers come from one ladder of squares; ZS = 0 takes any integer zeta.
 // The 2^(1 - zeta) factors are applied outside the pair loops (descriptor
 // sums and reverse-pass weights), a power-of-two scaling, so exact.
-// x^zeta, y^zeta (descriptor pass)
+// x^zeta (descriptor pass)
 template <class R, int ZS>
-__device__ __forceinline__ void zeta_pow(const BPParams &bp, R x, R y, R px[kBpZ], R py[kBpZ]) {
+__device__ __forceinline__ void zeta_pow(const BPParams &bp, P2<R> x, P2<R> p[kBpZ]) {
   if (ZS == 1) {
-    const R x2 = x * x, x4 = x2 * x2, x8 = x4 * x4;
-    const R y2 = y * y, y4 = y2 * y2, y8 = y4 * y4;
-    px[0] = x;
-    py[0] = y;
-    px[1] = x2;
-    py[1] = y2;
-    px[2] = x4;
-    py[2] = y4;
-    px[3] = x8 * x8;
-    py[3] = y8 * y8;
+    const P2<R> x2 = mul2(x, x), x4 = mul2(x2, x2), x8 = mul2(x4, x4);
+    p[0] = x;
+    p[1] = x2;
+    p[2] = x4;
+    p[3] = mul2(x8, x8);
   } else {
 #pragma unroll
-    for (int z = 0; z < kBpZ; ++z) {
-      ipow2<R>(x, y, bp.z_pow[z], px[z], py[z]);
-      px[z] *= x;
-      py[z] *= y;
-    }
+    for (int z = 0; z < kBpZ; ++z) p[z] = mul2(ipow2<R>(x, bp.z_pow[z]), x);
   }
 }
-// x^(zeta - 1), y^(zeta - 1) (reverse pass: A = x^(zeta-1) x, dA/dc = zeta x^(zeta-1))
+// x^(zeta - 1) (reverse pass: A = x^(zeta-1) x, dA/dc = zeta x^(zeta-1))
 template <class R, int ZS>
-__device__ __forceinline__ void zeta_pow_m1(const BPParams &bp, R x, R y, R px[kBpZ],
-                                            R py[kBpZ]) {
+__device__ __forceinline__ void zeta_pow_m1(const BPParams &bp, P2<R> x, P2<R> p[kBpZ]) {
   if (ZS == 1) {
-    const R x2 = x * x, x4 = x2 * x2, x8 = x4 * x4;
-    const R y2 = y * y, y4 = y2 * y2, y8 = y4 * y4;
-    px[0] = R(1);
-    py[0] = R(1);
-    px[1] = x;
-    py[1] = y;
-    px[2] = x2 * x;
-    py[2] = y2 * y;
-    px[3] = (x8 * x4) * (x2 * x);
-    py[3] = (y8 * y4) * (y2 * y);
+    const P2<R> x2 = mul2(x, x), x4 = mul2(x2, x2), x8 = mul2(x4, x4), x3 = mul2(x2, x);
+    p[0] = both(R(1));
+    p[1] = x;
+    p[2] = x3;
+    p[3] = mul2(mul2(x8, x4), x3);
   } else {
 #pragma unroll
-    for (int z = 0; z < kBpZ; ++z) ipow2<R>(x, y, bp.z_pow[z], px[z], py[z]);
+    for (int z = 0; z < kBpZ; ++z) p[z] = ipow2<R>(x, bp.z_pow[z]);
   }
 }
 
@@ -192,6 +199,9 @@ struct Slab {
   R *u4, *f4, *e;
   R *gax, *gay, *gaz, *gbx, *gby, *gbz;  // gradient sums (a side, b side)
   int *j;
+  uint16_t *row;                  // a round's neighbours, packed
+  uint16_t *queue;                // the lanes' pairs in the descriptor pass, [][32]; overlays
+                                  // the gradient sums, which are cleared after it
   R *G, *dG, *h1, *d1, *d2, *wc;  // wc: dE/dG of each angular slot
 };
 constexpr int kSlabFields = 14;   // per-neighbour reals besides e
@@ -214,16 +224,36 @@ __device__ __forceinline__ Q4<R> ld4(const R *p) {
 }
 // the exponentials of groups 2k and 2k + 1 at slot q
 template <class R>
-__device__ __forceinline__ void ld_e2(const R *e, int NB, int k, int q, R &e0, R &e1) {
+__device__ __forceinline__ P2<R> ld_e2(const R *e, int NB, int k, int q) {
   if constexpr (sizeof(R) == 4) {
     const float2 v = reinterpret_cast<const float2 *>(e + (size_t)2 * k * NB)[q];
-    e0 = v.x;
-    e1 = v.y;
+    return {v.x, v.y};
   } else {
     const double2 v = reinterpret_cast<const double2 *>(e + (size_t)2 * k * NB)[q];
-    e0 = v.x;
-    e1 = v.y;
+    return {v.x, v.y};
   }
+}
+
+// |u_b - u_a|^2 of two neighbours' pair vectors
+template <class R>
+__device__ __forceinline__ R sep2(const Q4<R> &a, const Q4<R> &b) {
+  const R sx = b.x - a.x, sy = b.y - a.y, sz = b.z - a.z;
+  return sx * sx + sy * sy + sz * sz;
+}
+// e^x of both components: 2^(x log2 e), results below the normal range flushed
+__device__ __forceinline__ P2<float> exp2v(P2<float> x) {
+  const P2<float> y = mul2(x, both(1.4426950408889634f));
+  P2<float> r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(y.x));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(y.y));
+  return r;
+}
+__device__ __forceinline__ P2<double> exp2v(P2<double> x) { return {exp(x.x), exp(x.y)}; }
+// exp(-eta R_ab^2) of (eta, kind) groups p and p + 1
+template <class R>
+__device__ __forceinline__ P2<R> gauss2(const BPParams &bp, int p, R rab2) {
+  return exp2v(mul2({pick<R>(bp.y_meta[p], bp.y_metaf[p]), pick<R>(bp.y_meta[p + 1], bp.y_metaf[p + 1])},
+                    both(rab2)));
 }
 
 constexpr int kVec = 80;  // >= kBpIn, a multiple of 16
@@ -250,12 +280,14 @@ __device__ __forceinline__ Slab<R> slab_at(char *base, int NB, int nY) {
   s.d2 = p + 2 * kVec + 64;
   s.wc = p + 2 * kVec + 96;
   s.j = reinterpret_cast<int *>(p + 2 * kVec + 96 + kBpSlots);
+  s.row = reinterpret_cast<uint16_t *>(s.j + NB);
+  s.queue = reinterpret_cast<uint16_t *>(s.gax);
   return s;
 }
 
 __host__ __device__ inline size_t slab_bytes(int NB, int nY, size_t rsz) {
   size_t b = rsz * ((size_t)(kSlabFields + nY) * NB + 2 * kVec + 96 + kBpSlots) +
-             sizeof(int) * (size_t)NB;
+             (sizeof(int) + sizeof(uint16_t)) * (size_t)NB;
   return (b + 15) / 16 * 16;
 }
 
@@ -296,8 +328,9 @@ constexpr int bp_blocks() {
 // NY: the (eta, kind) groups the kernel is compiled for (nY rounded up to an
 // even number); the padded groups carry zero exponentials, and slots without
 // a function zero weights, so the pair loops run without per-group guards.
-// ZS: the zeta set (zeta_pow).
-template <class P, bool ENERGY, int NY, int ZS>
+// ZS: the zeta set (zeta_pow).  K4: every group has kind 4 (the usual choice),
+// so only pairs inside R_c are evaluated and no group is asked for its kind.
+template <class P, bool ENERGY, int NY, int ZS, bool K4>
 __global__ void __launch_bounds__(bp_threads<P>(), bp_blocks<P>())
     k_bpnn(Sys s, BPParams bp, StepArgs a) {
   using GP = G<P>;
@@ -369,8 +402,6 @@ __global__ void __launch_bounds__(bp_threads<P>(), bp_blocks<P>())
       f[1] = R(0.5) * (cs + R(1));
       f[2] = half_pi_rc * sn;
       f[3] = R(0);
-      sl.gax[q] = sl.gay[q] = sl.gaz[q] = R(0);
-      sl.gbx[q] = sl.gby[q] = sl.gbz[q] = R(0);
 #pragma unroll
       for (int p = 0; p < NY; ++p)
         sl.e[(size_t)2 * (p >> 1) * NB + 2 * q + (p & 1)] =
@@ -397,9 +428,45 @@ __global__ void __launch_bounds__(bp_threads<P>(), bp_blocks<P>())
         accr[m] += v;
       }
   }
-  R acca[NS];
+  // sums of the slots (lambda = +1, -1) per (eta, kind) and zeta group; a slot
+  // without a function has zero weights, so its sum is never read
+  P2<R> acca[NS / 2];
 #pragma unroll
-  for (int m = 0; m < NS; ++m) acca[m] = 0;
+  for (int m = 0; m < NS / 2; ++m) acca[m] = both(R(0));
+  auto desc_pair = [&](const int qa, const int qb) {
+    const Q4<R> ua = ld4<R>(sl.u4 + 4 * qa), ub = ld4<R>(sl.u4 + 4 * qb);
+    const Q4<R> va = ld4<R>(sl.f4 + 4 * qa), vb = ld4<R>(sl.f4 + 4 * qb);
+    const R c = (ua.x * ub.x + ua.y * ub.y + ua.z * ub.z) * (va.x * vb.x);
+    const R rab2 = sep2(ua, ub);
+    const bool near = K4 || (bp.any4 && rab2 < rc2);
+    R fab = 0;
+    if (near) {
+      R sn, cs;
+      BM<R>::scpi(BM<R>::sq(rab2) * inv_rc, &sn, &cs);
+      fab = R(0.5) * (cs + R(1));
+    }
+    const R fab2 = va.y * vb.y;
+    P2<R> Y[NY / 2];
+#pragma unroll
+    for (int p = 0; p < NY; p += 2) {
+      P2<R> y = mul2(ld_e2<R>(sl.e, NB, p >> 1, qa), ld_e2<R>(sl.e, NB, p >> 1, qb));
+      y = mul2(y, both(fab2));
+      const P2<R> g = mul2(mul2(y, gauss2<R>(bp, p, rab2)), both(fab));
+      Y[p / 2] = K4 ? g
+                    : P2<R>{bp.y_kind[p] == 4 ? (near ? g.x : R(0)) : y.x,
+                            bp.y_kind[p + 1] == 4 ? (near ? g.y : R(0)) : y.y};
+    }
+    // (1 +- c)^zeta per zeta group (the factor 2^(1 - zeta) is applied to the sums)
+    P2<R> Pw[kBpZ];
+    zeta_pow<R, ZS>(bp, {R(1) + c, R(1) - c}, Pw);
+#pragma unroll
+    for (int p = 0; p < NY; ++p)
+#pragma unroll
+      for (int z = 0; z < kBpZ; ++z) {
+        P2<R> &q = acca[p * kBpZ + z];
+        q = fma2(Pw[z], both(p & 1 ? Y[p / 2].y : Y[p / 2].x), q);
+      }
+  };
   {
     const int npair = n * (n - 1) / 2;
     int qa = 0, rel = lane;  // pair t = (qa, qa + 1 + rel), rows in order of qa
@@ -407,57 +474,44 @@ __global__ void __launch_bounds__(bp_threads<P>(), bp_blocks<P>())
       rel -= n - 1 - qa;
       ++qa;
     }
-    for (int t = lane; t < npair; t += 32) {
-      const int qb = qa + 1 + rel;
-      const Q4<R> ua = ld4<R>(sl.u4 + 4 * qa), ub = ld4<R>(sl.u4 + 4 * qb);
-      const Q4<R> va = ld4<R>(sl.f4 + 4 * qa), vb = ld4<R>(sl.f4 + 4 * qb);
-      const R ax = ua.x, ay = ua.y, az = ua.z, fa = va.y;
-      const R bx = ub.x, by = ub.y, bz = ub.z, fb = vb.y;
-      const R c = (ax * bx + ay * by + az * bz) * (va.x * vb.x);
-      const R sx = bx - ax, sy = by - ay, sz = bz - az;
-      const R rab2 = sx * sx + sy * sy + sz * sz;
-      const bool near = bp.any4 && rab2 < rc2;
-      R fab = 0;
-      if (near) {
-        R sn, cs;
-        BM<R>::scpi(BM<R>::sq(rab2) * inv_rc, &sn, &cs);
-        fab = R(0.5) * (cs + R(1));
-      }
-      R Y[NY];
-#pragma unroll
-      for (int p = 0; p < NY; p += 2) {
-        R ea0, ea1, eb0, eb1;
-        ld_e2<R>(sl.e, NB, p >> 1, qa, ea0, ea1);
-        ld_e2<R>(sl.e, NB, p >> 1, qb, eb0, eb1);
-        Y[p] = ea0 * eb0;
-        Y[p + 1] = ea1 * eb1;
-      }
-      const R fab2 = fa * fb;
-#pragma unroll
-      for (int p = 0; p < NY; ++p) {
-        Y[p] *= fab2;
-        if (bp.y_kind[p] == 4)
-          Y[p] = near ? Y[p] * BM<R>::ex(-pick<R>(bp.y_eta[p], bp.y_etaf[p]) * rab2) * fab
-                      : R(0);
-      }
-      // (1 +- c)^zeta per zeta group (the factor 2^(1 - zeta) is applied to the sums)
-      R Pp[kBpZ], Pm[kBpZ];
-      zeta_pow<R, ZS>(bp, R(1) + c, R(1) - c, Pp, Pm);
-      // every slot of the used groups (a slot without a function has zero
-      // weights, so its sum is never read)
-#pragma unroll
-      for (int p = 0; p < NY; ++p)
-#pragma unroll
-        for (int z = 0; z < kBpZ; ++z) {
-          const int m = (p * kBpZ + z) * 2;
-          acca[m] += Pp[z] * Y[p];
-          acca[m + 1] += Pm[z] * Y[p];
-        }
+    auto advance = [&]() {
       rel += 32;
       while (qa < n - 1 && rel >= n - 1 - qa) {
         rel -= n - 1 - qa;
         ++qa;
       }
+    };
+    // queue entries: a and b in one word while neighbour numbers have 8 bits,
+    // in two beyond; win: pairs of a lane that fit
+    const bool wide = NB > 256;
+    const int win = (int)(6 * (size_t)NB * sizeof(R) / (32 * sizeof(uint16_t))) >> (wide ? 1 : 0);
+    for (int t0 = 0; t0 < npair; t0 += 32 * win) {
+      int cnt = 0;
+      for (int t = t0 + lane; t < min(npair, t0 + 32 * win); t += 32, advance()) {
+        const int qb = qa + 1 + rel;
+        if (!K4 || sep2(ld4<R>(sl.u4 + 4 * qa), ld4<R>(sl.u4 + 4 * qb)) < rc2) {
+          if (wide) {
+            sl.queue[64 * cnt + lane] = (uint16_t)qa;
+            sl.queue[64 * cnt + 32 + lane] = (uint16_t)qb;
+          } else {
+            sl.queue[32 * cnt + lane] = (uint16_t)(qa << 8 | qb);
+          }
+          ++cnt;
+        }
+      }
+      for (int e = 0; e < cnt; ++e) {
+        int a, b;
+        if (wide) {
+          a = sl.queue[64 * e + lane];
+          b = sl.queue[64 * e + 32 + lane];
+        } else {
+          const int q = sl.queue[32 * e + lane];
+          a = q >> 8;
+          b = q & 255;
+        }
+        desc_pair(a, b);
+      }
+      __syncwarp();
     }
   }
 #pragma unroll
@@ -465,16 +519,20 @@ __global__ void __launch_bounds__(bp_threads<P>(), bp_blocks<P>())
     if (m < nr) accr[m] = warp_sum(accr[m]);
 #pragma unroll
   for (int m = 0; m < NS; ++m)
-    if ((used >> m) & 1ull)
-      acca[m] = warp_sum(acca[m]) *
-                pick<R>(bp.z_coef[(m >> 1) % kBpZ], bp.z_coeff[(m >> 1) % kBpZ]);
+    if ((used >> m) & 1ull) {
+      R &v = m & 1 ? acca[m >> 1].y : acca[m >> 1].x;
+      v = warp_sum(v) * pick<R>(bp.z_coef[(m >> 1) % kBpZ], bp.z_coeff[(m >> 1) % kBpZ]);
+    }
   if (lane == 0) {
 #pragma unroll
     for (int m = 0; m < kBpRad; ++m) sl.G[m] = m < nr ? accr[m] : R(0);
 #pragma unroll
     for (int m = 0; m < kBpSlots; ++m)
-      sl.G[kBpRad + m] = (m < NS && ((used >> m) & 1ull)) ? acca[m < NS ? m : 0] : R(0);
+      sl.G[kBpRad + m] = (m < NS && ((used >> m) & 1ull))
+                             ? (m & 1 ? acca[(m < NS ? m : 0) >> 1].y : acca[(m < NS ? m : 0) >> 1].x)
+                             : R(0);
   }
+  for (int q = lane; q < 6 * NB; q += 32) sl.gax[q] = R(0);  // gax .. gbz
   __syncwarp();
 
   // ---- 3. the atomic network and its reverse pass -------------------------
@@ -525,29 +583,29 @@ __global__ void __launch_bounds__(bp_threads<P>(), bp_blocks<P>())
       const R iab = ia * ib;
       const R c = (ax * bx + ay * by + az * bz) * iab;
       const R sx = bx - ax, sy = by - ay, sz = bz - az;
-      const R rab2 = sx * sx + sy * sy + sz * sz;
-      const bool near = bp.any4 && rab2 < rc2;
+      const R rab2 = sep2(ua, ub);
+      const bool near = K4 || (bp.any4 && rab2 < rc2);
       R rab = 0, fab = 0, dfab = 0, irab = 0;
       if (near) {
         rab = BM<R>::sq(rab2);
+        irab = BM<R>::rcp(rab);
         R sn, cs;
         BM<R>::scpi(rab * inv_rc, &sn, &cs);
         fab = R(0.5) * (cs + R(1));
         dfab = half_pi_rc * sn;
-        irab = BM<R>::rcp(rab);
       }
       // per zeta group: A = (1 +- c)^zeta and dA/dc (2^(1 - zeta) is in the weights)
-      R Ap[kBpZ], Am[kBpZ], dAp[kBpZ], dAm[kBpZ];
-      R Qp[kBpZ], Qm[kBpZ];
-      zeta_pow_m1<R, ZS>(bp, R(1) + c, R(1) - c, Qp, Qm);
+      P2<R> A[kBpZ], dA[kBpZ];
+      {
+        const P2<R> x = {R(1) + c, R(1) - c};
+        P2<R> Q[kBpZ];
+        zeta_pow_m1<R, ZS>(bp, x, Q);
 #pragma unroll
-      for (int z = 0; z < kBpZ; ++z) {
-        const R zt = pick<R>(bp.z_zeta[z], bp.z_zetaf[z]);
-        const R pp = Qp[z], pm = Qm[z];
-        Ap[z] = pp * (R(1) + c);
-        Am[z] = pm * (R(1) - c);
-        dAp[z] = zt * pp;
-        dAm[z] = -zt * pm;
+        for (int z = 0; z < kBpZ; ++z) {
+          const R zt = pick<R>(bp.z_zeta[z], bp.z_zetaf[z]);
+          A[z] = mul2(Q[z], x);
+          dA[z] = mul2(Q[z], {zt, -zt});
+        }
       }
       // per (eta, kind) group: the functions' weighted sums S2 = sum w A,
       // S1 = sum w dA/dc, times the group's factor Y and its derivatives
@@ -557,37 +615,47 @@ __global__ void __launch_bounds__(bp_threads<P>(), bp_blocks<P>())
       //   gs = f_a f_b / R_ab sum_(G4 groups) S2 E2 X (f_ab' - 2 eta R_ab f_ab)
       // with E2 = exp(-eta (R_a^2 + R_b^2)), X = exp(-eta R_ab^2) and f_ab the R_ab
       // cutoff for G4 groups (0 beyond R_c), X = f_ab = 1 for G5 groups
-      R al = 0, bu = 0, bw = 0, gs = 0;
-      R ea[NY], eb[NY];
-#pragma unroll
-      for (int p = 0; p < NY; p += 2) {
-        ld_e2<R>(sl.e, NB, p >> 1, qa, ea[p], ea[p + 1]);
-        ld_e2<R>(sl.e, NB, p >> 1, qb, eb[p], eb[p + 1]);
-      }
       const R rfa = ra * fa, rfb = rb * fb, rfab = rab * fab;
+      P2<R> al2 = both(R(0)), bu2 = al2, bw2 = al2, gs2 = al2;
 #pragma unroll
-      for (int p = 0; p < NY; ++p) {  // padded groups: zero exponentials and weights
-        R S1 = 0, S2 = 0;
-        R wv[2 * kBpZ];  // the group's slots: (z, lambda = +1), (z, lambda = -1)
-        ld_group<R>(sl.wc + p * 2 * kBpZ, wv);
+      for (int p = 0; p < NY; p += 2) {  // padded groups: zero exponentials and weights
+        P2<R> S1, S2, w[kBpZ], t;
+        ld_group<R>(sl.wc + p * 2 * kBpZ, w);  // slots without a function have w = 0
+        t = mul2(w[0], A[0]);
 #pragma unroll
-        for (int z = 0; z < kBpZ; ++z) {  // slots without a function have w = 0
-          S2 += wv[2 * z] * Ap[z] + wv[2 * z + 1] * Am[z];
-          S1 += wv[2 * z] * dAp[z] + wv[2 * z + 1] * dAm[z];
+        for (int z = 1; z < kBpZ; ++z) t = fma2(w[z], A[z], t);
+        S2.x = t.x + t.y;
+        t = mul2(w[0], dA[0]);
+#pragma unroll
+        for (int z = 1; z < kBpZ; ++z) t = fma2(w[z], dA[z], t);
+        S1.x = t.x + t.y;
+        ld_group<R>(sl.wc + (p + 1) * 2 * kBpZ, w);
+        t = mul2(w[0], A[0]);
+#pragma unroll
+        for (int z = 1; z < kBpZ; ++z) t = fma2(w[z], A[z], t);
+        S2.y = t.x + t.y;
+        t = mul2(w[0], dA[0]);
+#pragma unroll
+        for (int z = 1; z < kBpZ; ++z) t = fma2(w[z], dA[z], t);
+        S1.y = t.x + t.y;
+        const P2<R> m2eta = {R(-2) * pick<R>(bp.y_eta[p], bp.y_etaf[p]),
+                             R(-2) * pick<R>(bp.y_eta[p + 1], bp.y_etaf[p + 1])};
+        P2<R> Ex = mul2(ld_e2<R>(sl.e, NB, p >> 1, qa), ld_e2<R>(sl.e, NB, p >> 1, qb));
+        P2<R> E4 = mul2(Ex, gauss2<R>(bp, p, rab2)), Exf;  // E4: kind 4 only
+        if (K4) {
+          Exf = mul2(E4, both(fab));
+        } else {
+          const bool k0 = bp.y_kind[p] == 4, k1 = bp.y_kind[p + 1] == 4;
+          E4 = {k0 && near ? E4.x : R(0), k1 && near ? E4.y : R(0)};
+          Exf = {k0 ? E4.x * fab : Ex.x, k1 ? E4.y * fab : Ex.y};
         }
-        const R m2eta = R(-2) * pick<R>(bp.y_eta[p], bp.y_etaf[p]);
-        R Ex = ea[p] * eb[p], Exf = Ex;
-        const bool k4 = bp.y_kind[p] == 4;
-        if (k4) {
-          Ex = near ? Ex * BM<R>::ex(R(0.5) * m2eta * rab2) : R(0);
-          Exf = Ex * fab;
-        }
-        al += S1 * Exf;
-        const R T = S2 * Exf;
-        bu += T * (m2eta * rfa + dfa);
-        bw += T * (m2eta * rfb + dfb);
-        if (k4) gs += S2 * Ex * (m2eta * rfab + dfab);
+        al2 = fma2(S1, Exf, al2);
+        const P2<R> T = mul2(S2, Exf);
+        bu2 = fma2(T, fma2(m2eta, both(rfa), both(dfa)), bu2);
+        bw2 = fma2(T, fma2(m2eta, both(rfb), both(dfb)), bw2);
+        gs2 = fma2(mul2(S2, E4), fma2(m2eta, both(rfab), both(dfab)), gs2);
       }
+      R al = al2.x + al2.y, bu = bu2.x + bu2.y, bw = bw2.x + bw2.y, gs = gs2.x + gs2.y;
       const R fab2 = fa * fb;
       al *= fab2;
       bu *= fb * ia;
@@ -605,36 +673,31 @@ __global__ void __launch_bounds__(bp_threads<P>(), bp_blocks<P>())
     };
     const bool even = (n & 1) == 0;
     const int kfull = (n - 1) / 2;  // shifts that pair all n neighbours
-    if (n >= 32) {
-      // flat schedule over (shift, a): 32 consecutive entries span at most two
-      // shifts with disjoint a ranges and disjoint b = a + shift ranges, so
-      // no lane of an instruction shares a neighbour's sums with another
-      const int T = kfull * n + (even ? n / 2 : 0);
-      int k = 1, qa = lane;
-      for (int t0 = 0; t0 < T; t0 += 32) {
-        if (t0 + lane < T) {
-          int qb = qa + k;
-          if (qb >= n) qb -= n;
-          grad_pair(qa, qb);
-        }
-        __syncwarp();
-        qa += 32;
-        if (qa >= n) {
-          qa -= n;
-          ++k;
-        }
-      }
-    } else {
-      for (int k = 1; k <= kfull + (even ? 1 : 0); ++k) {
-        const int na_k = k > kfull ? n / 2 : n;  // the last shift of an even n pairs each couple once
-        const int qa = lane;
+    const unsigned lower = (1u << lane) - 1u;
+    for (int k = 1; k <= kfull + (even ? 1 : 0); ++k) {
+      const int na_k = k > kfull ? n / 2 : n;  // the last shift of an even n pairs each couple once
+      // the round's pairs that count, packed: neighbours a in order
+      int cnt = 0;
+      for (int a0 = 0; a0 < na_k; a0 += 32) {
+        const int qa = a0 + lane;
+        bool take = false;
         if (qa < na_k) {
           int qb = qa + k;
           if (qb >= n) qb -= n;
-          grad_pair(qa, qb);
+          take = !K4 || sep2(ld4<R>(sl.u4 + 4 * qa), ld4<R>(sl.u4 + 4 * qb)) < rc2;
         }
-        __syncwarp();
+        const unsigned m = __ballot_sync(0xffffffffu, take);
+        if (take) sl.row[cnt + __popc(m & lower)] = (uint16_t)qa;
+        cnt += __popc(m);
       }
+      __syncwarp();
+      for (int e = lane; e < cnt; e += 32) {
+        const int qa = sl.row[e];
+        int qb = qa + k;
+        if (qb >= n) qb -= n;
+        grad_pair(qa, qb);
+      }
+      __syncwarp();
     }
   }
   // radial terms, then the scatter: -g to atom j_a, +g to atom i
@@ -711,14 +774,16 @@ int warps_for(int precision) { return precision == 0 ? 4 : 8; }
 
 }  // namespace
 
-// the compiled group count for nY groups: nY rounded up to an even number
-int ny_compiled(int nY) { return nY <= 2 ? 2 : (nY <= 4 ? 4 : (nY <= 6 ? 6 : 8)); }
+// the compiled group count of a model: its groups rounded up to an even number
+int ny_compiled(const BPParams &p) {
+  return p.any5 ? 8 : (p.nY <= 2 ? 2 : (p.nY <= 4 ? 4 : (p.nY <= 6 ? 6 : 8)));
+}
 
 size_t bpnn_smem_bytes(const BPParams &p, int precision, int nmax, int *warps) {
   const size_t rsz = precision == 0 ? 8 : 4;
   const int nW = kBpIn * p.H1 + p.H1 + p.H1 * p.H2 + 2 * p.H2;
   const size_t wbytes = ((size_t)nW * rsz + 15) / 16 * 16;
-  const size_t per = slab_bytes(nmax, ny_compiled(p.nY), rsz);
+  const size_t per = slab_bytes(nmax, ny_compiled(p), rsz);
   int w = warps_for(precision);
   while (w > 1 && wbytes + (size_t)w * per > 200 * 1024) --w;
   if (warps) *warps = w;
@@ -726,37 +791,43 @@ size_t bpnn_smem_bytes(const BPParams &p, int precision, int nmax, int *warps) {
 }
 
 namespace {
-template <class P, int NY, int ZS>
+// a model with G5 functions takes the instance of 8 groups (K4 = false)
+template <class P, int NY, int ZS, bool K4>
 cudaError_t smem_attr_one(int b) {
-  cudaError_t e = cudaFuncSetAttribute(k_bpnn<P, true, NY, ZS>,
+  cudaError_t e = cudaFuncSetAttribute(k_bpnn<P, true, NY, ZS, K4>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_bpnn<P, false, NY, ZS>,
+    e = cudaFuncSetAttribute(k_bpnn<P, false, NY, ZS, K4>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   return e;
 }
-template <class P, int NY>
+template <class P, int NY, bool K4>
 cudaError_t smem_attr_ny(int b) {
-  cudaError_t e = smem_attr_one<P, NY, 0>(b);
-  if (e == cudaSuccess) e = smem_attr_one<P, NY, 1>(b);
+  cudaError_t e = smem_attr_one<P, NY, 0, K4>(b);
+  if (e == cudaSuccess) e = smem_attr_one<P, NY, 1, K4>(b);
   return e;
 }
 template <class P>
 cudaError_t smem_attr(int b) {
-  cudaError_t e = smem_attr_ny<P, 2>(b);
-  if (e == cudaSuccess) e = smem_attr_ny<P, 4>(b);
-  if (e == cudaSuccess) e = smem_attr_ny<P, 6>(b);
-  if (e == cudaSuccess) e = smem_attr_ny<P, 8>(b);
+  cudaError_t e = smem_attr_ny<P, 2, true>(b);
+  if (e == cudaSuccess) e = smem_attr_ny<P, 4, true>(b);
+  if (e == cudaSuccess) e = smem_attr_ny<P, 6, true>(b);
+  if (e == cudaSuccess) e = smem_attr_ny<P, 8, true>(b);
+  if (e == cudaSuccess) e = smem_attr_ny<P, 8, false>(b);
   return e;
 }
 template <class P, bool EN, int ZS>
 void go_ny(const Sys &s, const BPParams &p, StepArgs a, int grid, int threads, size_t sm,
            cudaStream_t st) {
-  switch (ny_compiled(p.nY)) {
-    case 2: k_bpnn<P, EN, 2, ZS><<<grid, threads, sm, st>>>(s, p, a); break;
-    case 4: k_bpnn<P, EN, 4, ZS><<<grid, threads, sm, st>>>(s, p, a); break;
-    case 6: k_bpnn<P, EN, 6, ZS><<<grid, threads, sm, st>>>(s, p, a); break;
-    default: k_bpnn<P, EN, 8, ZS><<<grid, threads, sm, st>>>(s, p, a); break;
+  if (p.any5) {
+    k_bpnn<P, EN, 8, ZS, false><<<grid, threads, sm, st>>>(s, p, a);
+    return;
+  }
+  switch (ny_compiled(p)) {
+    case 2: k_bpnn<P, EN, 2, ZS, true><<<grid, threads, sm, st>>>(s, p, a); break;
+    case 4: k_bpnn<P, EN, 4, ZS, true><<<grid, threads, sm, st>>>(s, p, a); break;
+    case 6: k_bpnn<P, EN, 6, ZS, true><<<grid, threads, sm, st>>>(s, p, a); break;
+    default: k_bpnn<P, EN, 8, ZS, true><<<grid, threads, sm, st>>>(s, p, a); break;
   }
 }
 template <class P, bool EN>

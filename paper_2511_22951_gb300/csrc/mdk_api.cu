@@ -1023,8 +1023,10 @@ int mdk_set_potential_bpnn(mdk_ctx *c, double rc, int n_rad, const int *rad_kind
       y = p.nY++;
       p.y_eta[y] = eta;
       p.y_etaf[y] = (float)eta;
+      p.y_meta[y] = -eta;
+      p.y_metaf[y] = -(float)eta;
       p.y_kind[y] = k;
-      if (k == 4) p.any4 = 1;
+      (k == 4 ? p.any4 : p.any5) = 1;
     }
     for (int q = 0; q < p.nZ; ++q)
       if (p.z_zeta[q] == zeta) z = q;

@@ -301,15 +301,15 @@ constexpr int kBpH = 32;                   // units per hidden layer
 // words of the packed weight area (largest network)
 constexpr int kBpWords = kBpIn * kBpH + kBpH + kBpH * kBpH + 2 * kBpH;
 struct BPParams {
-  int n_rad, nY, nZ, H1, H2, any4;
+  int n_rad, nY, nZ, H1, H2, any4, any5;   // any4 / any5: some group has kind 4 / 5
   unsigned long long slot_mask;            // slots holding a function
   double rc, b3;
   float rcf, b3f;
   int rad_kind[kBpRad];
   double rad_p0[kBpRad], rad_p1[kBpRad];
   float rad_p0f[kBpRad], rad_p1f[kBpRad];
-  double y_eta[kBpY];
-  float y_etaf[kBpY];
+  double y_eta[kBpY], y_meta[kBpY];        // eta, -eta
+  float y_etaf[kBpY], y_metaf[kBpY];
   int y_kind[kBpY];                        // 4: with the R_jk factors, 5: without
   int zset;                                // 1: the zetas are among {1, 2, 4, 16}, group z
                                            // holding zeta = 1, 2, 4, 16; 0: any integers
