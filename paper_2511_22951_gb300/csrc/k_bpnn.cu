@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(bp_threads<P>(), bp_blocks<P>())
   using R = typename GP::R;
   using V = typename GP::V;
   extern __shared__ __align__(16) char smem[];
-  const int N = run_n(s.st);
+  const int N = run_n(s, a);
   const size_t Nc = s.N_cap;
   const int NB = s.nmax;
   const int nY = bp.nY, nr = bp.n_rad, H1 = bp.H1, H2 = bp.H2;

@@ -42,19 +42,11 @@ __device__ __forceinline__ bool full_on(const Sys &s) {
   return flag_on(s) && *(volatile int *)&s.st->full != 0;
 }
 
-__global__ void k_pre(Sys s, int count_step, int use_cond, cudaGraphConditionalHandle h) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// Window and build kind of the build that st->rebuild asks for (one thread).
+__device__ __forceinline__ void plan_build(const Sys &s, int count_step) {
   DevStatus *st = s.st;
-  if (st->abort) {  // stepping stopped at an overflowing build: nothing more
-    if (use_cond) cudaGraphSetConditional(h, 0u);
-    return;
-  }
   st->step_build = count_step;
   st->build_ovf = 0;
-  if (count_step) {
-    st->since_build += 1;
-    st->n_steps += 1;  // index of the force evaluation that follows (Langevin noise)
-  }
   if (s.rebuild_every > 0 && st->since_build >= s.rebuild_every) st->rebuild = 1;
   // the window acts at builds that stepping triggers, not at explicit builds
   st->win_active = (s.win_on && count_step && st->rebuild) ? 1 : 0;
@@ -68,10 +60,66 @@ __global__ void k_pre(Sys s, int count_step, int use_cond, cudaGraphConditionalH
   if (st->win_active) {
     st->key_xmax = dkey(-INFINITY);
     st->key_xmin = dkey(INFINITY);
-    st->win_cut = -INFINITY;
     st->win_insert = 0;
   }
+}
+
+__global__ void k_pre(Sys s, int count_step, int use_cond, cudaGraphConditionalHandle h) {
+  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  DevStatus *st = s.st;
+  if (st->abort) {  // stepping stopped at an overflowing build: nothing more
+    if (use_cond) cudaGraphSetConditional(h, 0u);
+    return;
+  }
+  if (count_step) {
+    st->since_build += 1;
+    st->n_steps += 1;  // index of the force evaluation that follows (Langevin noise)
+  }
+  plan_build(s, count_step);
   if (use_cond) cudaGraphSetConditional(h, st->rebuild ? 1u : 0u);
+}
+
+// The end of a captured loop body of `places` steps.  The steps up to the first
+// that triggered a build (or to the end of the body, of the loop or of the
+// fixed interval) are done, the places after it did nothing (run_n).  The
+// check and the conditional nodes cost once per body instead of once per step:
+// a step without a build 19.4 -> 11.3 us on 256 FP64 LJ atoms (its force pass
+// alone: 11.1), 21.2 -> 14.4 us on 32,000 mixed.  The next body reads the copy
+// that this one started from: after an odd e it is written again (by the
+// build, or by k_regather).
+__global__ void k_loop_head(Sys s, int places, cudaGraphConditionalHandle h,
+                            cudaGraphConditionalHandle loop) {
+  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  DevStatus *st = s.st;
+  const unsigned trig = st->trig;
+  st->trig = 0u;
+  if (st->abort) {
+    st->left = 0;
+    cudaGraphSetConditional(h, 0u);
+    cudaGraphSetConditional(loop, 0u);
+    return;
+  }
+  int e = min(places, st->left);
+  if (s.rebuild_every > 0) e = min(e, max(1, s.rebuild_every - st->since_build));
+  const unsigned m = trig & ((1u << e) - 1u);
+  if (m) {
+    e = __ffs(m);
+    st->rebuild = 1;
+  }
+  st->left -= e;
+  st->since_build += e;
+  st->n_steps += e;  // index of the force evaluation that follows
+  st->n_bodies += 1;
+  st->regather = e & 1;
+  plan_build(s, 1);
+  cudaGraphSetConditional(h, st->rebuild || st->regather ? 1u : 0u);
+  cudaGraphSetConditional(loop, st->left > 0 ? 1u : 0u);
+}
+
+__global__ void k_set_left(Sys s, int left) {
+  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  s.st->left = left;
+  s.st->trig = 0u;
 }
 
 // ---- moving window (Sec. "Moving window simulation"; rules in mdk.h) ----
@@ -1016,9 +1064,11 @@ __global__ void k_replay_filter_head(Sys s) {
 }
 
 // gather copy of the positions in x with the cells of the last build (the
-// expression of the step epilogue)
-template <class P>
+// expression of the step epilogue); ODD: only after a loop body that ended on
+// the other copy, and not after a full build, which has written this one
+template <class P, bool ODD>
 __global__ void __launch_bounds__(kBlk) k_regather(Sys s, typename P::vec4 *out) {
+  if (ODD && (!s.st->regather || full_on(s))) return;
   const int N = s.st->N;
   const size_t Nc = s.N_cap;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
@@ -1063,7 +1113,14 @@ void launch_rebuild_head(const Sys &s, int count_step, cudaGraphConditionalHandl
 
 int rebuild_chain_kernels(const Sys &s) { return 11 + (s.win_on ? 4 : 0) + (s.outer_on ? 4 : 0); }
 
-int launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_graph,
+void launch_loop_head(const Sys &s, int places, cudaGraphConditionalHandle h,
+                      cudaGraphConditionalHandle loop, cudaStream_t st) {
+  k_loop_head<<<1, 32, 0, st>>>(s, places, h, loop);
+}
+
+void launch_set_left(const Sys &s, int left, cudaStream_t st) { k_set_left<<<1, 32, 0, st>>>(s, left); }
+
+int launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_graph, int loop,
                         cudaStream_t st) {
   static int g_atom = 0, g_build = 0, g_cells = 0, g_filter = 0;
   if (g_atom == 0) {
@@ -1114,26 +1171,32 @@ int launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_gra
     else
       k_build_filter<false><<<gF, kBlk, 0, st>>>(s);
   }
+  if (loop) {
+    if (precision == 0)
+      k_regather<Fp64, true><<<gN, kBlk, 0, st>>>(s, (dvec4 *)s.pg[target_pg]);
+    else
+      k_regather<Mixed, true><<<gN, kBlk, 0, st>>>(s, (float4 *)s.pg[target_pg]);
+  }
   k_finish<<<1, 32, 0, st>>>(s, from_graph);
-  return rebuild_chain_kernels(s) - 1;
+  return rebuild_chain_kernels(s) - 1 + (loop ? 1 : 0);
 }
 
 void launch_rebuild(const Sys &s, int target_pg, int precision, int count_step, cudaStream_t st) {
   k_pre<<<1, 32, 0, st>>>(s, count_step, 0, 0);
-  launch_rebuild_body(s, target_pg, precision, 0, st);
+  launch_rebuild_body(s, target_pg, precision, 0, 0, st);
 }
 
 void launch_replay_filter(const Sys &s, int target_pg, int precision, cudaStream_t st) {
   k_replay_filter_head<<<1, 32, 0, st>>>(s);
-  launch_rebuild_body(s, target_pg, precision, 0, st);
+  launch_rebuild_body(s, target_pg, precision, 0, 0, st);
 }
 
 void launch_regather(const Sys &s, int target_pg, int precision, cudaStream_t st) {
   const int g = std::min(1024, nblk(s.N_cap > 0 ? s.N_cap : 1, kBlk));
   if (precision == 0)
-    k_regather<Fp64><<<g, kBlk, 0, st>>>(s, (dvec4 *)s.pg[target_pg]);
+    k_regather<Fp64, false><<<g, kBlk, 0, st>>>(s, (dvec4 *)s.pg[target_pg]);
   else
-    k_regather<Mixed><<<g, kBlk, 0, st>>>(s, (float4 *)s.pg[target_pg]);
+    k_regather<Mixed, false><<<g, kBlk, 0, st>>>(s, (float4 *)s.pg[target_pg]);
 }
 
 int scan_blocks_for(int n_buckets) { return (n_buckets + kScanTile - 1) / kScanTile; }

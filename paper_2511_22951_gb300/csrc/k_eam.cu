@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P>()) k_rho(Sys s, EAMPara
   using V = typename GP::V;
   using T1 = typename GP::Tab1;
   const T1 *rt = GP::tab1(ep);
-  const int N = run_n(s.st);
+  const int N = run_n(s, a);
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
   const R rc2 = sizeof(R) == 8 ? (R)ep.rc2 : (R)ep.rc2f;
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P, ENERGY>()) k_eam(Sys s,
     tab = GP::pr8(ep);  // one 32-byte record per interval
   else
     tab = GP::pr(ep);
-  const int N = run_n(s.st);
+  const int N = run_n(s, a);
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
   const V *__restrict__ pgf = (const V *)s.pgF;  // neighbours: offsets and F'

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(256, 2) k_rho_half(Sys s, EAMParams ep, StepAr
     rt = w;
     __syncthreads();
   }
-  const int N = run_n(s.st);
+  const int N = run_n(s, a);
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
   const R rc2 = sizeof(R) == 8 ? (R)ep.rc2 : (R)ep.rc2f;
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(256) k_embed(Sys s, EAMParams ep, StepArgs a) 
   using H = HalfAcc<P>;
   using R = typename GP::R;
   using V = typename GP::V;
-  const int N = run_n(s.st);
+  const int N = run_n(s, a);
   const size_t Nc = s.N_cap;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(256, 2) k_eam_half(Sys s, EAMParams ep, StepAr
     tab = w;
     __syncthreads();
   }
-  const int N = run_n(s.st);
+  const int N = run_n(s, a);
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
   const V *__restrict__ pgf = (const V *)s.pgF;  // neighbours: offsets and F'

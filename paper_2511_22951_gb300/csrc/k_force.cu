@@ -20,7 +20,7 @@ constexpr int kBlk = 256;
 // several mdk_step calls is bitwise the run in one call.
 template <class P>
 __global__ void __launch_bounds__(kBlk) k_kick_drift(Sys s, StepArgs a) {
-  const int N = run_n(s.st);
+  const int N = run_n(s, a);
   const int i = blockIdx.x * kBlk + threadIdx.x;
   if (i >= N) return;
   const size_t Nc = s.N_cap;

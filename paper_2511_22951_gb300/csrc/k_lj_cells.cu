@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(256, 4) k_lj_cells(Sys s, LJParams lp, StepArg
   __shared__ V tile[kCellWarps][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (c >= s.n_cells || s.st->abort) return;  // whole warps leave together
+  if (c >= s.n_cells || run_n(s, a) == 0) return;  // whole warps leave together
   const int b0 = s.cell_start[c], b1 = s.cell_start[c + 1];
   if (b0 >= b1) return;
   const size_t Nc = s.N_cap;

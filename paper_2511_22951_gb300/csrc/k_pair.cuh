@@ -509,7 +509,7 @@ __device__ __forceinline__ void drift_publish(const Sys &s, const StepArgs &a, i
   const bool trig = bad || d2 > s.half_skin2;
   const unsigned act = __activemask();
   const unsigned m = __ballot_sync(act, trig);
-  if (m && (threadIdx.x & 31) == (__ffs(m) - 1)) atomicOr(&s.st->rebuild, 1);
+  if (m && (threadIdx.x & 31) == (__ffs(m) - 1)) trigger_build(s, a);
   if (bad) atomicOr(&s.st->bits, kStNonfinite);
   const Grid &g = s.grid[inf >> 8];
   const uint32_t cc = s.cellc[i];
@@ -551,8 +551,8 @@ __device__ __forceinline__ void philox4x64(unsigned long long c[4], unsigned lon
 // path: the thermostat force is computed in FP32 (it
 // is noise and friction, on GB300's fast pipe), xi = (out >> 40) 2^-24.
 template <class P>
-__device__ __forceinline__ void langevin(const Sys &s, int i, uint32_t inf, double &Fx,
-                                         double &Fy, double &Fz) {
+__device__ __forceinline__ void langevin(const Sys &s, const StepArgs &a, int i, uint32_t inf,
+                                         double &Fx, double &Fy, double &Fz) {
   const size_t Nc = s.N_cap;
   const int type = inf & 15u;
   double g, sig, u[3] = {0.0, 0.0, 0.0};
@@ -573,7 +573,7 @@ __device__ __forceinline__ void langevin(const Sys &s, int i, uint32_t inf, doub
     u[2] = s.lang_u[r][2];
   }
   unsigned long long c[4] = {(unsigned long long)s.id[i],
-                             (unsigned long long)s.st->n_steps, 0ull, 0ull};
+                             step_index(s, a), 0ull, 0ull};
   philox4x64(c, s.lang_seed, 0ull);
   double *F[3] = {&Fx, &Fy, &Fz};
   if (sizeof(typename G<P>::R) == 8) {
@@ -608,7 +608,7 @@ __device__ __forceinline__ void epilogue64(const Sys &s, const StepArgs &a, int 
   }
   const int type = inf & 15u;
   const bool piston = (inf & kInfoPiston) != 0;
-  if ((s.n_lang > 0 || s.lang_rep_on) && !piston) langevin<P>(s, i, inf, Fx, Fy, Fz);
+  if ((s.n_lang > 0 || s.lang_rep_on) && !piston) langevin<P>(s, a, i, inf, Fx, Fy, Fz);
   const double c = 0.5 * a.dt * s.acc_over_m[type];
   double vx = s.v[i], vy = s.v[Nc + i], vz = s.v[2 * Nc + i];
   if (piston) {
@@ -647,8 +647,8 @@ __device__ __forceinline__ void epilogue64(const Sys &s, const StepArgs &a, int 
 // cell, both rounded from FP64: a few 1e-7 A against skin/2), except for
 // atoms flagged far, which keep the FP64 test.  This keeps GB300's slow FP64
 // pipe to the state updates themselves.
-__device__ __forceinline__ void langevin_f(const Sys &s, int i, uint32_t inf, float &Fx,
-                                           float &Fy, float &Fz) {
+__device__ __forceinline__ void langevin_f(const Sys &s, const StepArgs &a, int i, uint32_t inf,
+                                           float &Fx, float &Fy, float &Fz) {
   const size_t Nc = s.N_cap;
   const int type = inf & 15u;
   double g, sig, u[3] = {0.0, 0.0, 0.0};
@@ -669,7 +669,7 @@ __device__ __forceinline__ void langevin_f(const Sys &s, int i, uint32_t inf, fl
     u[2] = s.lang_u[r][2];
   }
   unsigned long long c[4] = {(unsigned long long)s.id[i],
-                             (unsigned long long)s.st->n_steps, 0ull, 0ull};
+                             step_index(s, a), 0ull, 0ull};
   philox4x64(c, s.lang_seed, 0ull);
   const float gf = (float)g, sigf = (float)sig;
   float *F[3] = {&Fx, &Fy, &Fz};
@@ -718,7 +718,7 @@ __device__ __forceinline__ void drift32(const Sys &s, const StepArgs &a, int i, 
   }
   const unsigned act = __activemask();
   const unsigned m = __ballot_sync(act, trig);
-  if (m && (threadIdx.x & 31) == (__ffs(m) - 1)) atomicOr(&s.st->rebuild, 1);
+  if (m && (threadIdx.x & 31) == (__ffs(m) - 1)) trigger_build(s, a);
   if (bad) atomicOr(&s.st->bits, kStNonfinite);
   float4 *out = (float4 *)s.pg[a.cur ^ 1];
   out[i] = make_float4(px, py, pz, __uint_as_float(inf));
@@ -742,7 +742,7 @@ __device__ __forceinline__ void epilogue32(const Sys &s, const StepArgs &a, int 
   }
   const int type = inf & 15u;
   const bool piston = (inf & kInfoPiston) != 0;
-  if ((s.n_lang > 0 || s.lang_rep_on) && !piston) langevin_f(s, i, inf, Fx, Fy, Fz);
+  if ((s.n_lang > 0 || s.lang_rep_on) && !piston) langevin_f(s, a, i, inf, Fx, Fy, Fz);
   const double dx = kick32(s, a, type, Fx), dy = kick32(s, a, type, Fy),
                dz = kick32(s, a, type, Fz);
   double vx = __ldcs(s.v + i), vy = __ldcs(s.v + Nc + i), vz = __ldcs(s.v + 2 * Nc + i);

@@ -92,17 +92,19 @@ struct mdk_ctx {
   // pass of that step
   bool pending = false;
   LaunchCfg cfg;  // pair-kernel launch shape (mdk_autotune)
-  // CUDA graphs of two plain steps, one per parity of the gather copy
+  // CUDA graphs, one per parity of the gather copy: [0] the rebuild chain
+  // after one step, [1] a loop of plain steps
   bool graphs_on = true;
   cudaStream_t cap_stream = nullptr;
-  cudaGraphExec_t gexec[2] = {nullptr, nullptr};
-  uint64_t gkey[2] = {0, 0};
+  cudaGraphExec_t gexec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+  uint64_t gkey[2][2] = {{0, 0}, {0, 0}};
   cudaStream_t body_stream = nullptr;  // captures the conditional rebuild bodies
-  int64_t graph_kernels = 0;  // kernels of one graph that run at every replay
+  int64_t loop_kernels = 0;   // kernels of one loop body that run every time
+  int64_t body_kernels = 0;   // kernels of one conditional rebuild body
+  long long graph_builds0 = 0;  // device counts of in-graph builds and loop
+  long long bodies0 = 0;        // bodies at mdk_profile
   double *ctr_dev = nullptr;     // cell-centre tables in the workspace
   std::vector<double> ctr_host;  // their values (kept until the upload completes)
-  int64_t body_kernels = 0;   // kernels of one conditional rebuild body
-  long long graph_builds0 = 0;  // device count of in-graph builds at mdk_profile
   // moving window
   bool win_on = false;
   double win_L_behind = 0.0, win_L_ahead = 0.0, win_slab_lx = 0.0, win_gap = 0.0,
@@ -485,6 +487,8 @@ __global__ void k_init_status(Sys s, int N) {
     st->step_build = 0;
     st->build_ovf = 0;
     st->rebuild = 1;
+    st->trig = 0;
+    st->left = 0;
     st->bits = 0;
     st->max_nnbr = 0;
     st->since_build = 0;
@@ -577,8 +581,8 @@ int timed(mdk_ctx *c, std::vector<std::pair<int, int>> &log, int n_kernels, F la
   return cudaPeekAtLastError() == cudaSuccess ? MDK_OK : MDK_ERR_CUDA;
 }
 
-int force_pass(mdk_ctx *c, Mode mode, int energy, double dt) {
-  StepArgs a{dt, c->cur, energy, (float)(0.5 * dt)};
+int force_pass(mdk_ctx *c, Mode mode, int energy, double dt, int pos = -1) {
+  StepArgs a{dt, c->cur, energy, (float)(0.5 * dt), 0, pos};
   const bool cells = c->pot == 1 && c->cfg.half == 2;
   const bool half = (c->pot == 1 || c->pot == 2) && c->cfg.half == 1;
   const int nk = c->pot == 1 ? (half ? 2 : 1) : (c->pot == 2 && half ? 4 : 2);
@@ -717,10 +721,16 @@ uint64_t graph_key(const mdk_ctx *c, double dt) {
   return h;
 }
 
-// The rebuild chain of a captured step: the head kernel (k_pre) decides and
-// sets the value of an IF conditional node whose body holds the rest of the
-// chain, so a step without a rebuild runs two kernels, not the whole chain.
-int capture_conditional_chain(mdk_ctx *c) {
+// Steps that one loop body holds.  A place after a triggered build does
+// nothing, but its blocks still start and exit (~1 us for a small grid, ~60 us
+// for 65,000 blocks), and a build comes about every ten steps.
+int loop_places(const mdk_ctx *c) { return c->N_cap * (int64_t)c->cfg.tpa <= (1 << 22) ? 8 : 2; }
+
+// The rebuild chain of captured steps: the head kernel (k_pre, or k_loop_head
+// after a loop body) decides and sets the value of an IF conditional node
+// whose body holds the rest of the chain, so steps without a rebuild run one
+// kernel, not the whole chain.
+int capture_conditional_chain(mdk_ctx *c, int places, cudaGraphConditionalHandle loop) {
   cudaStreamCaptureStatus cs;
   cudaGraph_t g = nullptr;
   const cudaGraphNode_t *deps = nullptr;
@@ -728,8 +738,10 @@ int capture_conditional_chain(mdk_ctx *c) {
   MDK_CK(cudaStreamGetCaptureInfo(c->cap_stream, &cs, nullptr, &g, nullptr, nullptr, nullptr));
   cudaGraphConditionalHandle h;
   MDK_CK(cudaGraphConditionalHandleCreate(&h, g, 0, 0));
-  launch_rebuild_head(c->sys, 1, h, c->cap_stream);
-  c->launches += 1;
+  if (places > 0)
+    launch_loop_head(c->sys, places, h, loop, c->cap_stream);
+  else
+    launch_rebuild_head(c->sys, 1, h, c->cap_stream);
   MDK_CK(cudaPeekAtLastError());
   MDK_CK(cudaStreamGetCaptureInfo(c->cap_stream, &cs, nullptr, &g, &deps, nullptr, &nd));
   cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
@@ -743,50 +755,96 @@ int capture_conditional_chain(mdk_ctx *c) {
   cudaGraph_t body = cp.conditional.phGraph_out[0];
   MDK_CK(cudaStreamBeginCaptureToGraph(c->body_stream, body, nullptr, nullptr, 0,
                                        cudaStreamCaptureModeThreadLocal));
-  c->body_kernels = launch_rebuild_body(c->sys, c->cur, c->precision, 1, c->body_stream);
+  c->body_kernels =
+      launch_rebuild_body(c->sys, c->cur, c->precision, 1, places > 0, c->body_stream);
   const cudaError_t e = cudaPeekAtLastError();
   cudaGraph_t out = nullptr;
   MDK_CK(cudaStreamEndCapture(c->body_stream, &out));
   return e == cudaSuccess ? MDK_OK : MDK_ERR_CUDA;
 }
 
-// Capture two plain steps (force pass + rebuild chain, twice) starting from
-// gather-copy parity `parity`; the graph ends at the same parity.
-int capture_two_steps(mdk_ctx *c, int parity, double dt, uint64_t key) {
+// The graph of one kind for gather-copy parity `parity` (both end at it):
+//  kind 0: the rebuild chain after a step on its own;
+//  kind 1: a WHILE node whose body holds loop_places steps (force passes that
+//    take turns with the two gather copies) and the chain; st->left steps in all.
+int ensure_graph(mdk_ctx *c, int kind, int parity, double dt, uint64_t key) {
+  if (c->gexec[kind][parity] && c->gkey[kind][parity] == key) return MDK_OK;
   if (!c->cap_stream) MDK_CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
   if (!c->body_stream) MDK_CK(cudaStreamCreateWithFlags(&c->body_stream, cudaStreamNonBlocking));
-  const cudaStream_t keep_stream = c->stream;
-  const int keep_cur = c->cur;
-  const bool keep_prof = c->prof;
-  const int64_t keep_launches = c->launches;
-  MDK_CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-  c->stream = c->cap_stream;
-  c->cur = parity;
-  c->prof = false;
+  cudaGraph_t top = nullptr, inner = nullptr;
+  MDK_CK(cudaGraphCreate(&top, 0));
+  cudaGraphConditionalHandle loop{};
   int r = MDK_OK;
-  for (int h = 0; h < 2 && !r; ++h) {
-    r = force_pass(c, kStep, 0, dt);
-    c->cur ^= 1;
-    if (!r) r = capture_conditional_chain(c);
+  const int places = kind == 1 ? loop_places(c) : 0;
+  if (kind == 1) {
+    cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
+    cudaGraphNode_t node;
+    cudaError_t e = cudaGraphConditionalHandleCreate(&loop, top, 1, cudaGraphCondAssignDefault);
+    cp.conditional.handle = loop;
+    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.size = 1;
+    if (e == cudaSuccess) e = cudaGraphAddNode(&node, top, nullptr, nullptr, 0, &cp);
+    if (e == cudaSuccess)
+      inner = cp.conditional.phGraph_out[0];
+    else
+      r = MDK_ERR_CUDA;
+  } else {
+    inner = top;
   }
-  c->stream = keep_stream;
-  c->cur = keep_cur;
-  c->prof = keep_prof;
-  c->graph_kernels = c->launches - keep_launches;
-  c->launches = keep_launches;
-  cudaGraph_t g = nullptr;
-  const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
-  if (r || e != cudaSuccess || !g) {
-    if (g) cudaGraphDestroy(g);
+  if (!r && cudaStreamBeginCaptureToGraph(c->cap_stream, inner, nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeThreadLocal) != cudaSuccess)
+    r = MDK_ERR_CUDA;
+  if (!r) {
+    const cudaStream_t keep_stream = c->stream;
+    const int keep_cur = c->cur;
+    const bool keep_prof = c->prof;
+    const int64_t keep_launches = c->launches;
+    c->stream = c->cap_stream;
+    c->cur = parity;
+    c->prof = false;
+    for (int p = 0; p < places && !r; ++p) {
+      r = force_pass(c, kStep, 0, dt, p);
+      c->cur ^= 1;
+    }
+    if (places > 0) c->loop_kernels = c->launches - keep_launches + 1;
+    if (!r) r = capture_conditional_chain(c, places, loop);
+    c->stream = keep_stream;
+    c->cur = keep_cur;
+    c->prof = keep_prof;
+    c->launches = keep_launches;
+    cudaGraph_t out = nullptr;
+    if (cudaStreamEndCapture(c->cap_stream, &out) != cudaSuccess && !r) r = MDK_ERR_CUDA;
+  }
+  if (!r) {
+    if (c->gexec[kind][parity]) cudaGraphExecDestroy(c->gexec[kind][parity]);
+    c->gexec[kind][parity] = nullptr;
+    if (cudaGraphInstantiate(&c->gexec[kind][parity], top, 0) != cudaSuccess) r = MDK_ERR_CUDA;
+  }
+  cudaGraphDestroy(top);
+  if (r) {
     cudaGetLastError();
-    return r ? r : MDK_ERR_CUDA;
+    return r;
   }
-  if (c->gexec[parity]) cudaGraphExecDestroy(c->gexec[parity]);
-  c->gexec[parity] = nullptr;
-  const cudaError_t ei = cudaGraphInstantiate(&c->gexec[parity], g, 0);
-  cudaGraphDestroy(g);
-  if (ei != cudaSuccess) return MDK_ERR_CUDA;
-  c->gkey[parity] = key;
+  c->gkey[kind][parity] = key;
+  return MDK_OK;
+}
+
+// whether a call steps with graphs: not while profiling, and not while the
+// caller captures the stream (the steps then go into that graph one by one)
+bool use_graphs(mdk_ctx *c) {
+  if (!c->graphs_on || c->prof) return false;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) cudaGetLastError();
+  return cs == cudaStreamCaptureStatusNone;
+}
+
+// the rebuild chain after a step on its own (counted)
+int step_chain(mdk_ctx *c, bool graphs, double dt, uint64_t key) {
+  if (!graphs) return rebuild_chain(c, 1);
+  const int r = ensure_graph(c, 0, c->cur, dt, key);
+  if (r) return r;
+  MDK_CK(cudaGraphLaunch(c->gexec[0][c->cur], c->stream));
+  c->launches += 1;
   return MDK_OK;
 }
 
@@ -872,8 +930,8 @@ int mdk_create(mdk_ctx **out, const double box_lo[3], const double box_hi[3],
 int mdk_destroy(mdk_ctx *c) {
   if (!c) return MDK_ERR_BAD_ARG;
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
-  for (int q = 0; q < 2; ++q)
-    if (c->gexec[q]) cudaGraphExecDestroy(c->gexec[q]);
+  for (int q = 0; q < 4; ++q)
+    if (c->gexec[q / 2][q % 2]) cudaGraphExecDestroy(c->gexec[q / 2][q % 2]);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->body_stream) cudaStreamDestroy(c->body_stream);
   delete c;
@@ -1696,6 +1754,8 @@ int mdk_step(mdk_ctx *c, double dt, int64_t nsteps) {
     if (r) return r;
   }
   Sys &s = c->sys;
+  const bool graphs = use_graphs(c);
+  const uint64_t key = graphs ? graph_key(c, dt) : 0;
   if (c->pending) {
     // a restored mid-step state: its first half-kick, drift and list build
     // are done; the steps start with the pending force pass
@@ -1712,24 +1772,26 @@ int mdk_step(mdk_ctx *c, double dt, int64_t nsteps) {
     r = timed(c, c->ev_kick, 1, [&] { launch_kick_drift(s, c->precision, a, c->stream); });
     if (r) return r;
     c->cur ^= 1;
-    r = rebuild_chain(c, 1);
+    r = step_chain(c, graphs, dt, key);
     if (r) return r;
   }
-  const uint64_t key = c->graphs_on ? graph_key(c, dt) : 0;
   auto is_thermo = [&](int64_t q) {
     return c->thermo_every > 0 && ((c->steps_done + q) % c->thermo_every) == 0;
   };
   for (int64_t q = 1; q <= nsteps; ++q) {
-    // two plain steps (neither the last nor a thermo step) run as one graph
-    if (c->graphs_on && !c->prof && q + 1 < nsteps && !is_thermo(q) && !is_thermo(q + 1)) {
+    // runs of plain steps (neither the last nor a thermo step) go into one loop
+    if (graphs && q + 1 < nsteps && !is_thermo(q) && !is_thermo(q + 1)) {
+      int64_t run = nsteps - q;  // q .. nsteps - 1
+      if (c->thermo_every > 0)
+        run = std::min<int64_t>(run, c->thermo_every - 1 - (c->steps_done + q - 1) % c->thermo_every);
+      run = std::min<int64_t>(run, 1 << 30);
       const int par = c->cur;
-      if (!c->gexec[par] || c->gkey[par] != key) {
-        r = capture_two_steps(c, par, dt, key);
-        if (r) return r;
-      }
-      MDK_CK(cudaGraphLaunch(c->gexec[par], c->stream));
-      c->launches += c->graph_kernels;
-      ++q;  // the graph ran steps q and q + 1; the parity is back to par
+      r = ensure_graph(c, 1, par, dt, key);
+      if (r) return r;
+      launch_set_left(s, (int)run, c->stream);
+      MDK_CK(cudaGraphLaunch(c->gexec[1][par], c->stream));
+      c->launches += 1;
+      q += run - 1;  // the loop ends at the parity it started from
       continue;
     }
     const int64_t gstep = c->steps_done + q;
@@ -1746,7 +1808,7 @@ int mdk_step(mdk_ctx *c, double dt, int64_t nsteps) {
     }
     if (!last) {
       c->cur ^= 1;
-      r = rebuild_chain(c, 1);
+      r = step_chain(c, graphs, dt, key);
       if (r) return r;
     }
   }
@@ -1984,6 +2046,7 @@ int mdk_profile(mdk_ctx *c, int enable) {
     int r = read_status(c, &st);
     if (r) return r;
     c->graph_builds0 = st.n_graph_builds;
+    c->bodies0 = st.n_bodies;
   }
   c->prof = enable != 0;
   c->ev_used = 0;
@@ -2014,10 +2077,10 @@ int mdk_get_profile(mdk_ctx *c, double *out) {
   out[1] = (double)c->ev_force.size();
   out[2] = total(c->ev_chain);
   out[3] = (double)c->ev_chain.size();
-  // kernels launched: those enqueued directly, those of every graph replay,
-  // and the rebuild bodies that the graphs' conditional nodes ran
-  out[4] = (double)c->launches + (double)c->body_kernels * (double)(st.n_graph_builds -
-                                                                     c->graph_builds0);
+  // kernels launched: those enqueued directly (and the graphs' heads), those of
+  // the loop bodies and those of the rebuild bodies that conditional nodes ran
+  out[4] = (double)c->launches + (double)c->loop_kernels * (double)(st.n_bodies - c->bodies0) +
+           (double)c->body_kernels * (double)(st.n_graph_builds - c->graph_builds0);
   out[5] = (double)st.n_builds;
   out[6] = total(c->ev_kick);
   out[7] = (double)c->ev_kick.size();

@@ -54,10 +54,17 @@ struct DevStatus {
                          // the state stays that of the moment of the build
                          // (positions drifted, velocities at the half step)
   int rebuild;           // != 0: rebuild the lists before the next force pass
+  // captured steps: bit p set: the step at place p of the loop body moved an
+  // atom past skin/2, so the places after it wait for the list build; left:
+  // steps the loop still has to do at the body's start
+  unsigned trig;
+  int left;
+  int regather;          // the body ended on the other gather copy
   unsigned bits;         // kSt* raised since the host last cleared them
   int max_nnbr;          // longest list seen at a build
   long long n_builds;
   long long n_graph_builds;  // builds run inside a captured step's conditional node
+  long long n_bodies;        // loop bodies run
   long long n_steps;
   int since_build;       // steps since the last build
   int next_id;           // id of the next atom a moving window appends
@@ -81,11 +88,6 @@ struct DevStatus {
   int step_build;        // this build was triggered by stepping (k_pre, count_step)
   int build_ovf;         // a list of this build outgrew its capacity
 };
-
-// atoms a force or integration kernel works on: none once stepping aborted
-__device__ __forceinline__ int run_n(const DevStatus *st) {
-  return st->abort ? 0 : st->N;
-}
 
 // one replica's box and cell grid
 struct Grid {
@@ -451,22 +453,53 @@ struct StepArgs {
   int cur;              // gather copy read this step (pg[cur]); pg[cur^1] written
   int energy;           // compute per-atom energies / virials this step
   float hdtf;           // dt / 2 in FP32 (mixed-path kicks)
-  int f32;              // k_kick_drift: the force pass in use ends its steps with
+  int f32 = 0;          // k_kick_drift: the force pass in use ends its steps with
                         // FP32 forces (the mixed full-list kernels), so the first
                         // kick takes the FP32 increment of the stored force
+  int pos = -1;         // place in the captured loop body, -1: a step on its own
 };
+
+// atoms a force or integration kernel works on: none once stepping aborted,
+// and none where the step at a.pos of a loop body has to wait -- an earlier
+// one triggered a list build, the loop has fewer steps left, or the
+// fixed-interval build is due
+__device__ __forceinline__ int run_n(const Sys &s, const StepArgs &a) {
+  const DevStatus *st = s.st;
+  bool wait = st->abort != 0;
+  if (a.pos >= 0) {
+    wait = wait || a.pos >= st->left || (st->trig & ((1u << a.pos) - 1u)) != 0u;
+    if (s.rebuild_every > 0 && a.pos > 0) wait = wait || st->since_build + a.pos >= s.rebuild_every;
+  }
+  return wait ? 0 : st->N;
+}
+// an atom moved past skin/2: the lists are rebuilt before the next step
+__device__ __forceinline__ void trigger_build(const Sys &s, const StepArgs &a) {
+  if (a.pos < 0)
+    atomicOr(&s.st->rebuild, 1);
+  else
+    atomicOr(&s.st->trig, 1u << a.pos);
+}
+// index of this force evaluation (Langevin noise)
+__device__ __forceinline__ unsigned long long step_index(const Sys &s, const StepArgs &a) {
+  return (unsigned long long)(s.st->n_steps + (a.pos > 0 ? a.pos : 0));
+}
 
 void launch_rebuild(const Sys &s, int target_pg, int precision, int count_step, cudaStream_t st);
 // checkpoint restore: a filter build (two-level lists) at the positions in x,
 // and the gather copy pg[target_pg] of x with the cells of the last build
 void launch_replay_filter(const Sys &s, int target_pg, int precision, cudaStream_t st);
 void launch_regather(const Sys &s, int target_pg, int precision, cudaStream_t st);
-// The same chain in two parts for a captured step: the head decides whether
+// The same chain in two parts for captured steps: the head decides whether
 // to rebuild and sets the conditional node's value; the body (run by that
 // node only when the value is 1) rebuilds.  Returns the kernels of the body.
 void launch_rebuild_head(const Sys &s, int count_step, cudaGraphConditionalHandle h,
                          cudaStream_t st);
-int launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_graph,
+// the head after a loop body of `places` steps: counts the steps done and sets
+// the loop's condition too
+void launch_loop_head(const Sys &s, int places, cudaGraphConditionalHandle h,
+                      cudaGraphConditionalHandle loop, cudaStream_t st);
+void launch_set_left(const Sys &s, int left, cudaStream_t st);
+int launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_graph, int loop,
                         cudaStream_t st);
 int rebuild_chain_kernels(const Sys &s);
 void launch_set_piston(const Sys &s, const uint8_t *flags, int64_t n_flags, cudaStream_t st);
