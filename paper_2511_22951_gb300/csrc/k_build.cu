@@ -9,7 +9,7 @@
 // (no host round trip to decide whether to rebuild):
 //   k_pre       count steps since the last build; fixed-interval trigger
 //   k_bin       wrap periodic coordinates, cell id per atom, cell histogram
-//   k_scan_*    exclusive scan of the histogram (3 phases)
+//   k_scan_*    exclusive scan of the histogram (3 phases; one at small sizes)
 //   k_scatter   counting-sort scatter into cell order (atomic slots)
 //   k_cell_sort order each cell's atoms by their permanent id (determinism)
 //   k_permute   gather every per-atom array into the new order (scratch)
@@ -330,6 +330,35 @@ __device__ __forceinline__ int block_exscan(int v, int *total) {
   return res;
 }
 
+// ONE: the whole scan in this kernel, where one tile holds all buckets (the
+// partials' two launches, ~2.5 us each, are what the scan costs then)
+template <bool ONE>
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(Sys s) {
+  if (!full_on(s)) return;
+  const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
+  int loc[kScanItems];
+  int sum = 0;
+#pragma unroll
+  for (int q = 0; q < kScanItems; ++q) {
+    loc[q] = (base + q <= s.n_cells) ? s.cell_cnt[base + q] : 0;
+    sum += loc[q];
+  }
+  __shared__ int tot;
+  int pre = block_exscan(sum, &tot) + (ONE ? 0 : s.scan_part[blockIdx.x]);
+#pragma unroll
+  for (int q = 0; q < kScanItems; ++q) {
+    const int c = base + q;
+    if (c <= s.n_cells) {
+      s.cell_start[c] = pre;
+      s.cell_fill[c] = pre;
+      s.cell_cnt[c] = 0;  // ready for the next build
+    }
+    pre += loc[q];
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kScanThreads - 1)
+    s.cell_start[s.n_cells + 1] = pre;
+}
+
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(Sys s) {
   if (!full_on(s)) return;
   const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
@@ -361,32 +390,6 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_top(Sys s) {
     if (base + q < s.n_scan_blocks) s.scan_part[base + q] = pre;
     pre += loc[q];
   }
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(Sys s) {
-  if (!full_on(s)) return;
-  const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
-  int loc[kScanItems];
-  int sum = 0;
-#pragma unroll
-  for (int q = 0; q < kScanItems; ++q) {
-    loc[q] = (base + q <= s.n_cells) ? s.cell_cnt[base + q] : 0;
-    sum += loc[q];
-  }
-  __shared__ int tot;
-  int pre = block_exscan(sum, &tot) + s.scan_part[blockIdx.x];
-#pragma unroll
-  for (int q = 0; q < kScanItems; ++q) {
-    const int c = base + q;
-    if (c <= s.n_cells) {
-      s.cell_start[c] = pre;
-      s.cell_fill[c] = pre;
-      s.cell_cnt[c] = 0;  // ready for the next build
-    }
-    pre += loc[q];
-  }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kScanThreads - 1)
-    s.cell_start[s.n_cells + 1] = pre;
 }
 
 __global__ void __launch_bounds__(kBlk) k_scatter(Sys s) {
@@ -1111,7 +1114,9 @@ void launch_rebuild_head(const Sys &s, int count_step, cudaGraphConditionalHandl
   k_pre<<<1, 32, 0, st>>>(s, count_step, 1, h);
 }
 
-int rebuild_chain_kernels(const Sys &s) { return 11 + (s.win_on ? 4 : 0) + (s.outer_on ? 4 : 0); }
+int rebuild_chain_kernels(const Sys &s) {
+  return (s.n_scan_blocks == 1 ? 9 : 11) + (s.win_on ? 4 : 0) + (s.outer_on ? 4 : 0);
+}
 
 void launch_loop_head(const Sys &s, int places, cudaGraphConditionalHandle h,
                       cudaGraphConditionalHandle loop, cudaStream_t st) {
@@ -1145,9 +1150,13 @@ int launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_gra
     k_win_insert<<<gN, kBlk, 0, st>>>(s);
   }
   k_bin<<<gN, kBlk, 0, st>>>(s);
-  k_scan_reduce<<<s.n_scan_blocks, kScanThreads, 0, st>>>(s);
-  k_scan_top<<<1, kScanThreads, 0, st>>>(s);
-  k_scan_apply<<<s.n_scan_blocks, kScanThreads, 0, st>>>(s);
+  if (s.n_scan_blocks == 1) {
+    k_scan_apply<true><<<1, kScanThreads, 0, st>>>(s);
+  } else {
+    k_scan_reduce<<<s.n_scan_blocks, kScanThreads, 0, st>>>(s);
+    k_scan_top<<<1, kScanThreads, 0, st>>>(s);
+    k_scan_apply<false><<<s.n_scan_blocks, kScanThreads, 0, st>>>(s);
+  }
   k_scatter<<<gN, kBlk, 0, st>>>(s);
   k_cell_sort<<<gC, kBlk, 0, st>>>(s);
   if (precision == 0)
