@@ -79,32 +79,39 @@ __device__ __forceinline__ void scatter(double2 *acc, int k, double a0, double a
 struct Fx64 {
   unsigned *lo;
   int *hi;
-  __device__ __forceinline__ void add(int slot, long long v) const {
-    const unsigned vl = (unsigned)v;
-    int vh = (int)(v >> 32);
+  __device__ __forceinline__ void add(int slot, unsigned vl, int vh) const {
     const unsigned old = atomicAdd(lo + slot, vl);
     if (old + vl < old) vh += 1;
     if (vh != 0) atomicAdd(hi + slot, vh);
+  }
+  __device__ __forceinline__ void add(int slot, double w) const {
+    const long long v = __double2ll_rn(w);
+    add(slot, (unsigned)v, (int)(v >> 32));
+  }
+  // A float rounded to 64 bits without the conversion to int64, which runs on
+  // GB300's FP64 pipe (16 cycles of an SM per warp; 8 conversions a pair kept
+  // that pipe 89% busy): the high word by an FMA at 1.5 2^23 (|w| < 2^53, see
+  // k_adj_scale), the exact rest (at most 2^31 in magnitude) to 32 bits.
+  // k_adj_pair on the 143,460-atom cold-curve batch 243 -> 183 us.
+  __device__ __forceinline__ void add(int slot, float w) const {
+    const float m = fmaf(w, 0x1p-32f, 12582912.0f);
+    const int vl = __float2int_rn(fmaf(m - 12582912.0f, -0x1p32f, w));
+    add(slot, (unsigned)vl, __float_as_int(m) - 0x4B400000 + (vl >> 31));
   }
   __device__ __forceinline__ long long get(int slot) const {
     return (long long)(((unsigned long long)(unsigned)hi[slot] << 32) | lo[slot]);
   }
 };
 
-// value * S rounded to an integer, in the pair precision (S is a power of
-// two, so the product is exact; FP64 work per pair is what the FP32 pair
-// arithmetic of the mixed path avoids on GB300's slow FP64 pipe)
-__device__ __forceinline__ long long to_fx(float v, float S) { return __float2ll_rn(v * S); }
-__device__ __forceinline__ long long to_fx(double v, double S) { return __double2ll_rn(v * S); }
-
 // fixed-point add of cv * (value weights) + cd * (derivative weights) to the
 // slots (y_k, M_k, y_{k+1}, M_{k+1}) = 2k .. 2k + 3
 template <class R>
 __device__ __forceinline__ void scatter_fx(const Fx64 &h, int k, R S, R a0, R a1, R a2, R a3) {
-  h.add(2 * k, to_fx(a0, S));
-  h.add(2 * k + 1, to_fx(a1, S));
-  h.add(2 * k + 2, to_fx(a2, S));
-  h.add(2 * k + 3, to_fx(a3, S));
+  // S is a power of two, so the products are exact
+  h.add(2 * k, a0 * S);
+  h.add(2 * k + 1, a1 * S);
+  h.add(2 * k + 2, a2 * S);
+  h.add(2 * k + 3, a3 * S);
 }
 
 // add a block's shared histogram to the global one (zeros skipped)
@@ -265,7 +272,9 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_c(Sys s, EAMParams ep, AdjArg
 }
 
 // ---- the fixed-point scale of pass pair (one thread) ---------------------------------
-__global__ void k_adj_scale(Sys s, EAMParams ep, AdjArgs a) {
+// fp32: the mixed path's terms also stay below 2^53 (Fx64::add; a limit for
+// systems of a few atoms only, where P B would allow more)
+__global__ void k_adj_scale(Sys s, EAMParams ep, AdjArgs a, int fp32) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const double gE = __longlong_as_double(a.aux[0]), gF = __longlong_as_double(a.aux[1]);
   const double lam = __longlong_as_double(a.aux[2]), fp = __longlong_as_double(a.aux[3]);
@@ -274,6 +283,7 @@ __global__ void k_adj_scale(Sys s, EAMParams ep, AdjArgs a) {
   double S = 1.0;
   if (P * B > 0.0 && isfinite(P * B)) {
     int e = 61 - (int)ceil(log2(P * B));
+    if (fp32) e = min(e, 52 - (int)ceil(log2(B)));
     e = e > 100 ? 100 : (e < -100 ? -100 : e);  // a finite FP32 scale too
     S = ldexp(1.0, e);
   }
@@ -431,7 +441,7 @@ int run(const Sys &s, const EAMParams &ep, const double *gF, AdjArgs a, int64_t 
   const int N = (int)n_atoms;
   k_adj_load<P><<<nblk(s.N_cap > 0 ? s.N_cap : 1, 256), 256, 0, st>>>(s, gF, a);
   k_adj_c<P><<<persistent_grid(k_adj_c<P>, b_c, N), kAdjBlock, b_c, st>>>(s, ep, a);
-  k_adj_scale<<<1, 32, 0, st>>>(s, ep, a);
+  k_adj_scale<<<1, 32, 0, st>>>(s, ep, a, sizeof(typename GP::R) == 4);
   k_adj_pair<P><<<persistent_grid(k_adj_pair<P>, b_p, N), kAdjBlock, b_p, st>>>(s, ep, a);
   k_adj_fin<<<nblk(2 * ep.nr + ep.nrho, 256), 256, 0, st>>>(ep, a);
   return 0;
