@@ -143,6 +143,17 @@ int mdk_set_potential_eam(mdk_ctx *ctx, int nr, double rc, const double *phi,
                           const double *F);
 
 /*
+ * New knot values for the tables of mdk_set_potential_eam, from device arrays
+ * on the context's stream (a fitting loop's parameters stay on the GPU: no
+ * host copy, no synchronisation).  Same nr and nrho as before, with a
+ * workspace set; otherwise MDK_ERR_ORDER and nothing changes (use
+ * mdk_set_potential_eam).  rc and rho_max may change.  Results are those of
+ * mdk_set_potential_eam with the same values.
+ */
+int mdk_update_eam_knots(mdk_ctx *ctx, int nr, double rc, const double *phi, const double *rho,
+                         int nrho, double rho_max, const double *F);
+
+/*
  * Behler-Parrinello neural-network potential (Sec. "Molecular dynamics with
  * Behler-Parrinello neural networks"), single element: E = sum_i E_i, E_i
  * from atom i's network applied to its symmetry functions over the

@@ -223,8 +223,15 @@ __device__ __forceinline__ double hslope(const double *y, int n, int k) {
 }
 
 __global__ void k_eam_prepare(int nr, int nrho, double rc, const double *phi, const double *rho,
-                              const double *F, EAMTablesDev o) {
+                              const double *F, EAMTablesDev o, double *keep) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (keep != phi) {
+    if (k < nr) {
+      keep[k] = phi[k];
+      keep[nr + k] = rho[k];
+    }
+    if (k < nrho) keep[2 * nr + k] = F[k];
+  }
   if (k < nr) {
     const double mp = hslope(phi, nr, k), mr = hslope(rho, nr, k);
     o.phi64[k] = make_double2(phi[k], mp);
@@ -378,9 +385,10 @@ void launch_eam_rho(const Sys &s, const EAMParams &p, int precision, StepArgs a,
 }
 
 void launch_eam_prepare(const EAMParams &p, const double *phi, const double *rho,
-                        const double *F, EAMTablesDev out, cudaStream_t st) {
+                        const double *F, EAMTablesDev out, double *keep, cudaStream_t st) {
   const int n = p.nr > p.nrho ? p.nr : p.nrho;
-  k_eam_prepare<<<nblk(n, 256), 256, 0, st>>>(p.nr, p.nrho, p.rc, phi, rho, F, out);
+  k_eam_prepare<<<nblk(n, 256), 256, 0, st>>>(p.nr, p.nrho, p.rc, phi, rho, F, out,
+                                              keep);
 }
 
 }  // namespace mdk

@@ -535,8 +535,10 @@ void launch_kick_drift(const Sys &s, int precision, StepArgs a, cudaStream_t st)
 // per-replica sums into s.red, and E [n_rep] / virial [n_rep][6] (device) unless
 // null; returns the number of kernels launched
 int launch_reduce(const Sys &s, int with_ke, double *E, double *virial, cudaStream_t st);
+// the device tables from knots on the device; keep: the workspace's own copy of
+// the knots, [nr | nr | nrho] (may be where they come from)
 void launch_eam_prepare(const EAMParams &p, const double *phi, const double *rho,
-                        const double *F, EAMTablesDev out, cudaStream_t st);
+                        const double *F, EAMTablesDev out, double *keep, cudaStream_t st);
 // the far records at index N_cap of both gather copies (see pad_entry)
 void launch_init_far(const Sys &s, int precision, cudaStream_t st);
 void launch_load_state(const Sys &s, const double *x_aos, const double *v_aos,

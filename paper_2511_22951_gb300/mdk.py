@@ -54,6 +54,7 @@ SIGNATURES = {
     "mdk_set_capacity": [_P, _I64],
     "mdk_set_potential_lj": [_P, _D, _D, _D, _I],
     "mdk_set_potential_eam": [_P, _I, _D, _P, _P, _I, _D, _P],
+    "mdk_update_eam_knots": [_P, _I, _D, _P, _P, _I, _D, _P],
     "mdk_set_potential_bpnn": [_P, _D, _I, _P, _P, _I, _P, _P, _I, _I, _P, _P, _P, _P, _P, _D],
     "mdk_workspace_size": [_P, ctypes.POINTER(_SZ)],
     "mdk_set_workspace": [_P, _P, _SZ],
@@ -227,6 +228,19 @@ class Context:
                "mdk_set_potential_eam")
         self._eam_sizes = (phi.shape[0], F.shape[0])
         self.version += 1
+
+    def update_eam_knots(self, phi, rho, F, rc, rho_max):
+        """New knot values of the current tables from float64 CUDA tensors of
+        the same sizes, enqueued on the context's stream.  False (and nothing
+        changed) when the sizes differ or no workspace is set yet: then
+        set_potential_eam is the call."""
+        r = self.lib.mdk_update_eam_knots(self.h, phi.shape[0], rc, _ptr(phi), _ptr(rho),
+                                          F.shape[0], rho_max, _ptr(F))
+        if r == MDK_ERR_ORDER:
+            return False
+        _check(r, "mdk_update_eam_knots")
+        self.version += 1
+        return True
 
     def set_potential_bpnn(self, model):
         """Behler-Parrinello model (workloads.BPNNModel-like: rc, rad_kind,
