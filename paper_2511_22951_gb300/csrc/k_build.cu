@@ -22,6 +22,8 @@
 
 #include <algorithm>
 
+#include <climits>
+
 #include "mdk_internal.cuh"
 
 namespace mdk {
@@ -553,8 +555,11 @@ struct ListOut {
 //
 // The candidates of a cell are its 27 template cells' atoms in template order,
 // flattened: candidate p sits in the range whose cumulative length passes p,
-// so every chunk of 32 candidates is full whatever the cells hold.  Phase 1:
-// lane l loads candidate p (cells are contiguous runs of atoms), shifts it by
+// so every chunk of 32 candidates is full whatever the cells hold.  Phase 0:
+// candidates farther than r_ns from the bounding box of the slice's atoms are
+// left out, the others packed into the tile in their order (a distance to a
+// box per candidate instead of one to every atom of the slice).
+// Phase 1: a lane loads one of them, shifts it by
 // its stencil offset and tests it against every atom of the slice,
 //   r^2 - r_ns^2 = (c.c - r_ns^2) + p.p - 2 c.p,
 // two atoms per packed FP32 instruction with their constants broadcast from
@@ -572,11 +577,14 @@ struct ListOut {
 // arithmetic per atom and cell, one shared store per candidate, lanes of two
 // cells diverging).  Phase 2 with a lane per mask word and a scan of their bit
 // counts was slower: the accepted candidates sit in few, dense words.
-// Measured (ncu, one launch, before -> now): 388,204 argon atoms (529 candidates,
-// 78 neighbours) 305 -> 213 us (653 -> 335 warp instructions per atom, issue
-// active 77% -> 55%: the two phases' shared-memory chains take turns with
-// the packed tests); 8,388,608 atoms with the outer list (890 candidates, 136
-// entries) 9.1 -> 6.0 ms; 256 atoms 57 -> 21 us, 32,000 71 -> 46 us.
+// Measured (ncu, one launch; that version -> lanes over candidates -> phase 0
+// added): 388,204 argon atoms (529 candidates, 78 neighbours) 305 -> 213 ->
+// 204 us; 442,368 atoms of 64 replicas of densities up to twice that (cells up
+// to 10 A wide, up to ~1500 candidates) 510 -> 379 us; 8,388,608 atoms with the
+// outer list (890 candidates, 136 entries) 9.1 -> 5.65 -> 5.12 ms; 640,000
+// slab atoms 305 -> 290 us; 256 atoms 57 -> 21 -> 19 us, 32,000 71 -> 46 -> 43
+// us.  A box of a cell of about r_ns keeps ~70% of the candidates, of a cell
+// 1.15 times as wide ~60%.
 //
 // Error of the FP32 test: atoms in their cells (|p_d| <= 0.6 h) give |c| <=
 // 2.8 h, each product and sum rounds to 2^-24 of at most 15 h^2, so r^2 is off
@@ -584,9 +592,12 @@ struct ListOut {
 // (|p_d| <= 2 h) give 75 h^2 and 2.5e-5 h^2.  Candidates within a band four
 // times that wide (Sys.build_band = 2e-5 h^2, and five times it) take the
 // exact FP64 test of the definition, and so do far atoms (NaN offsets).
+// The distance to the box is a difference of rounded coordinates: its square is
+// off by less than 2e-6 h^2 in cells, 1e-5 h^2 with clamped atoms, and phase 0
+// takes what is within r_ns^2 + 1e-4 h^2; a slice with a far atom has no box.
 // Lists come out in the order of the candidates: template cell, then atom.
 constexpr int kBWarps = 4;     // warps per block
-constexpr int kTileCh = 32;    // chunks of 32 candidates per tile (two phases per tile)
+constexpr int kTileCh = 32;    // chunks of 32 candidates per tile (the three phases per tile)
 // Atoms of a slice at most, by the size of the system: short slices give a
 // small system more warps (a warp's chain of dependent loads and shared
 // reads takes ~10 us whatever its slice holds), long ones share the loading
@@ -601,8 +612,20 @@ struct BuildWarp {
   float4 sh[28];                   // template cell: shift s h, entry code in .w
   int end[28];                     // end of the template cell's candidates (flattened)
   int off[28];                     // atom = candidate + off
+  int self[32];                    // where the slice's own atoms sit in the tile (-1: not in it)
   uint8_t chunk[kTileCh][32];      // phase 2: chunk of an atom's w-th nonzero mask word
 };
+
+constexpr uint32_t kNoEntry = 0xffffffffu;  // stencil code 63: no candidate has it
+
+// floats in the order of signed integers (NaN past the infinities)
+__device__ __forceinline__ int ordered_int(float v) {
+  const int b = __float_as_int(v);
+  return b ^ ((b >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float ordered_float(int b) {
+  return __int_as_float(b ^ ((b >> 31) & 0x7fffffff));
+}
 
 template <bool HALF>
 __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, int slice_max) {
@@ -664,8 +687,6 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
         if (lane >= o) incl += t;
       }
       const int total = __shfl_sync(full, incl, 31);
-      // this lane's atom among the flattened candidates (template cell 13 is its own)
-      const int own = a0 + lane - __shfl_sync(full, first - (incl - len), 13);
       const float bx = 0.6f * g.hf[0], by = 0.6f * g.hf[1], bz = 0.6f * g.hf[2];
       // in its cell (false for NaN too)
       auto inside = [&](const float4 &p) {
@@ -678,6 +699,7 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
         sm.off[lane] = first - (incl - len);
       }
       bool out_a = false, far_a = false;
+      float lo[3], hi[3];  // the slice's bounding box
       {
         float4 p = make_float4(0.f, 0.f, 0.f, 1e30f);  // no atom: far from everything
         if (lane < n) {
@@ -685,6 +707,12 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
           out_a = !inside(p);
           p.w = fmaf(p.z, p.z, fmaf(p.y, p.y, p.x * p.x));
           far_a = !(p.w == p.w);
+        }
+        const float pd[3] = {p.x, p.y, p.z};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          lo[d] = ordered_float(__reduce_min_sync(full, lane < n ? ordered_int(pd[d]) : INT_MAX));
+          hi[d] = ordered_float(__reduce_max_sync(full, lane < n ? ordered_int(pd[d]) : INT_MIN));
         }
         float *q = reinterpret_cast<float *>(&sm.a0[lane >> 1]) + (lane & 1);
         q[0] = -2.f * p.x;
@@ -694,24 +722,74 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
         q[2] = p.w;
       }
       __syncwarp();
-      int t = 0;      // this lane's template cell (moves up with its candidates)
+      const float mx = 0.5f * (lo[0] + hi[0]), my = 0.5f * (lo[1] + hi[1]), mz = 0.5f * (lo[2] + hi[2]);
+      const float wx = 0.5f * (hi[0] - lo[0]), wy = 0.5f * (hi[1] - lo[1]), wz = 0.5f * (hi[2] - lo[2]);
+      const float cull = __any_sync(full, far_a) ? INFINITY : mid + 5.0f * s.build_band;
+      int t_tile = 0;  // this lane's template cell (moves up with its candidates)
       int count = 0;  // this lane's atom
-      for (int tile = 0; tile < total; tile += 32 * kTileCh) {
-        const int n_ch = min(kTileCh, (total - tile + 31) >> 5);
+      int next_p = 0;
+      for (bool one = true; next_p < total; one = false) {
+        // ---- phase 0: the tile's candidates, those within reach of the box -
+        int slots = 0;
+        sm.self[lane] = -1;
+        __syncwarp();
+        int t = t_tile;
+        float4 rn[2];  // the records of the next 64 candidates, loaded ahead
+        int jn[2], tn[2];
+        auto look = [&](int base_p) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int p = base_p + 32 * h + lane;
+            tn[h] = -1;
+            if (p < total) {
+              while (p >= sm.end[t]) ++t;
+              tn[h] = t;
+              jn[h] = dbg_idx(s, p + sm.off[t], s.N_cap);
+              rn[h] = __ldg(s.pf + jn[h]);
+            }
+          }
+        };
+        look(next_p);
+        for (; next_p < total && slots <= 32 * kTileCh - 64; next_p += 64) {
+          const float4 r[2] = {rn[0], rn[1]};
+          const int jc[2] = {jn[0], jn[1]}, tc[2] = {tn[0], tn[1]};
+          t_tile = t;
+          look(next_p + 64);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            bool in = tc[h] >= 0;
+            uint32_t code = 0;
+            if (in) {
+              const float4 d = sm.sh[tc[h]];
+              code = __float_as_uint(d.w);
+              const float gx = fmaxf(fabsf(r[h].x + d.x - mx) - wx, 0.0f);
+              const float gy = fmaxf(fabsf(r[h].y + d.y - my) - wy, 0.0f);
+              const float gz = fmaxf(fabsf(r[h].z + d.z - mz) - wz, 0.0f);
+              // a far atom (NaN offsets) is within reach of everything
+              in = !(fmaf(gz, gz, fmaf(gy, gy, gx * gx)) > cull) || !(r[h].x == r[h].x);
+            }
+            const unsigned b = __ballot_sync(full, in);
+            const int at = slots + __popc(b & ((1u << lane) - 1u));
+            if (in) {
+              sm.ent[at] = code | ((uint32_t)jc[h] << 6);
+              if (code == 21u && (unsigned)(jc[h] - a0) < (unsigned)n) sm.self[jc[h] - a0] = at;
+            }
+            slots += __popc(b);
+          }
+        }
+        __syncwarp();
+        const int n_ch = (slots + 31) >> 5;
         // ---- phase 1: two chunks of 32 candidates at a time ---------------
         float4 r2[2];  // the records of the next pair of chunks, loaded ahead
-        int j2[2], t2[2];
+        uint32_t e2[2];
         auto fetch = [&](int c) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            const int p = tile + 32 * (c + h) + 31 - lane;
-            if (c < n_ch && p < total) {
-              while (p >= sm.end[t]) ++t;
-              t2[h] = t;
-              j2[h] = dbg_idx(s, p + sm.off[t], s.N_cap);
-              r2[h] = __ldg(s.pf + j2[h]);
-            } else {
-              t2[h] = -1;
+            const int p = 32 * (c + h) + 31 - lane;
+            e2[h] = kNoEntry;
+            if (p < slots) {
+              e2[h] = sm.ent[p];
+              r2[h] = __ldg(s.pf + nbr_j(e2[h]));
             }
           }
         };
@@ -723,23 +801,22 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             q[h] = make_float4(0.f, 0.f, 0.f, 1e30f);
-            e[h] = 0;
-            if (t2[h] >= 0) {
-              const float4 r = r2[h], d = sm.sh[t2[h]];
-              e[h] = __float_as_uint(d.w) | ((uint32_t)j2[h] << 6);
+            e[h] = e2[h];
+            if (e[h] != kNoEntry) {
+              const float4 r = r2[h];
+              const float4 d = sm.sh[(e[h] & 3u) + 3u * ((e[h] >> 2) & 3u) + 9u * ((e[h] >> 4) & 3u)];
               const float x = r.x + d.x, y = r.y + d.y, z = r.z + d.z;
               q[h] = make_float4(x, y, z, fmaf(z, z, fmaf(y, y, x * x)) - mid);
               out_c = out_c || !inside(r);
               far_c = far_c || !(r.x == r.x);
             }
-            sm.ent[32 * (c + h) + lane] = e[h];
           }
           fetch(c + 2);
           float near = 1e30f;  // smallest distance of a test from r_ns^2
           auto keep = [&](int k, uint32_t ent) {
             return !HALF || half_keep(a0 + k, nbr_j(ent), (ent & 63u) > 21u);
           };
-#pragma unroll 2
+#pragma unroll 4
           for (int k = 0; k < n; k += 2) {
             const float4 u = sm.a0[k >> 1], v = sm.a1[k >> 1];
             unsigned b[4];
@@ -766,7 +843,7 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
               for (int h = 0; h < 2; ++h) {
                 const float d2 = fmaf(q[h].z, v[0], fmaf(q[h].y, u[2], fmaf(q[h].x, u[0], q[h].w + v[2])));
                 bool acc = d2 < -width;
-                if (!acc && !(d2 > width) && tile + 32 * (c + h) + 31 - lane < total)
+                if (!acc && !(d2 > width) && e[h] != kNoEntry)
                   acc = exact_pair(s, g, a0 + k, e[h], c0, c1, c2, lo_.rns2);
                 const unsigned b = __ballot_sync(full, acc && keep(k, e[h]));
                 if (lane == 0)
@@ -779,7 +856,7 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
         // an atom is no neighbour of itself (its images are)
         uint32_t *mw = reinterpret_cast<uint32_t *>(sm.mask) + 4 * (lane >> 1) + (lane & 1);
         auto word = [](int c) { return (c >> 1) * 64 + 2 * (c & 1); };
-        const int self = own - tile;
+        const int self = sm.self[lane];
         if (lane < n && (unsigned)self < (unsigned)(32 * n_ch))
           mw[word(self >> 5)] &= ~(0x80000000u >> (self & 31));
         // ---- phase 2: this lane's atom takes its accepted entries ----------
@@ -803,14 +880,14 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
             ent = sm.ent + 32 * sm.chunk[at][lane];
             ++at;
           }
-          const int b = 31 - __clz(m);
-          const uint32_t e = ent[max(b, 0)];
+          const int z = __clz(m);
+          const uint32_t e = ent[min(z, 31)];
           const bool some = m != 0;
-          m ^= some ? 1u << b : 0u;
+          m ^= some ? 0x80000000u >> z : 0u;
           return some ? e : pad_entry(Nc);
         };
         const int most = __reduce_max_sync(full, add);
-        if (tile == 0) {
+        if (one) {
           for (int k = 0; k < most; k += kGroup) {
             uint32_t w[kGroup];
 #pragma unroll
