@@ -530,14 +530,45 @@ __device__ __noinline__ bool exact_pair(const Sys &s, const Grid &g, int i, uint
   return r2 < rns2;
 }
 
-// Half lists keep each unordered pair in one of its two atoms' lists: for
-// j != i in the list of the smaller index when i + j is even and of the
-// larger when it is odd (so every atom keeps about half of its neighbours,
-// whatever its place in the cell order).  (i, j, s) and (j, i, -s) pass the
-// same distance test, so the half list is exactly one of each mirror pair.
-__device__ __forceinline__ bool half_keep(int i, int j, bool s_pos) {
-  if (j == i) return s_pos;
-  return (i < j) == (((i ^ j) & 1) == 0);
+// Half lists keep each unordered pair in one of its two atoms' lists: of the
+// atom that lies behind along a fixed direction w, of the smaller index (or,
+// for an image of the atom itself, the positive stencil offset) where both lie
+// level.  In a solid every neighbour at d has one at about -d, so all atoms
+// keep the same number (39 of 78 in argon, where the lanes of a warp walk
+// their lists together); a parity rule on the indices left 39 +- 4, and a
+// warp walked its longest, 48.  w is a direction along which no vector of a
+// cubic lattice up to 4.3 half lattice constants is level (0.098 of one at
+// least, 0.049 for simple cubic).  The place along w is an integer of the
+// atom's record and the shifts are odd integers of the stencil offset, so
+// (i, j, s) and (j, i, -s) decide alike whatever the rounding: the half list
+// is exactly one of each mirror pair.  Both passed the same distance test.
+struct HalfKey {
+  float kx, ky, kz;  // units per A: 2^20 for a cell's extent along w
+  int sx, sy, sz;    // a cell's extents
+  __device__ __forceinline__ explicit HalfKey(const Grid &g) {
+    const float wx = -0.1488063f, wy = 0.7473134f, wz = -0.6475951f;
+    const float u = 1048576.0f / (fabsf(wx) * g.hf[0] + wy * g.hf[1] + fabsf(wz) * g.hf[2]);
+    kx = wx * u;
+    ky = wy * u;
+    kz = wz * u;
+    sx = __float2int_rn(kx * g.hf[0]);
+    sy = __float2int_rn(ky * g.hf[1]);
+    sz = __float2int_rn(kz * g.hf[2]);
+  }
+  // an atom's place along w (the integer in the low bits of 1.5 2^23 + p.w; 0
+  // for a far atom, whose offsets are NaN)
+  __device__ __forceinline__ int at(const float4 &p) const {
+    const float f = __fmaf_rn(p.z, kz, __fmaf_rn(p.y, ky, __fmaf_rn(p.x, kx, 12582912.0f)));
+    return f == f ? __float_as_int(f) : 0;
+  }
+  __device__ __forceinline__ int shift(uint32_t code) const {
+    return nbr_s(code, 0) * sx + nbr_s(code, 1) * sy + nbr_s(code, 2) * sz;
+  }
+};
+__device__ __forceinline__ bool half_keep(int i, int at_i, uint32_t code, int at_j) {
+  const int j = nbr_j(code);
+  const bool level = j == i ? (code & 63u) > 21u : i < j;
+  return at_i != at_j ? at_i < at_j : level;
 }
 
 // where a build writes: the Verlet list (s.nbr), or with the outer list on
@@ -612,6 +643,7 @@ struct BuildWarp {
   float4 sh[28];                   // template cell: shift s h, entry code in .w
   int end[28];                     // end of the template cell's candidates (flattened)
   int off[28];                     // atom = candidate + off
+  int key[32];                     // HALF: places of the slice's atoms along w
   int self[32];                    // where the slice's own atoms sit in the tile (-1: not in it)
   uint8_t chunk[kTileCh][32];      // phase 2: chunk of an atom's w-th nonzero mask word
 };
@@ -663,6 +695,7 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
       const int a0 = base + l0, n = __shfl_sync(full, n_sl, l0);
       const uint32_t cc = s.cellc[a0];
       const Grid &g = s.grid[s.info[a0] >> 8];
+      const HalfKey hk(g);
       const int c0 = cell_coord(cc, 0), c1 = cell_coord(cc, 1), c2 = cell_coord(cc, 2);
       // ---- the candidates: 27 runs of atoms, flattened --------------------
       int len = 0, first = 0;
@@ -705,6 +738,7 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
         if (lane < n) {
           p = __ldg(s.pf + a0 + lane);
           out_a = !inside(p);
+          if (HALF) sm.key[lane] = hk.at(p);
           p.w = fmaf(p.z, p.z, fmaf(p.y, p.y, p.x * p.x));
           far_a = !(p.w == p.w);
         }
@@ -797,6 +831,7 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
         for (int c = 0; c < n_ch; c += 2) {
           float4 q[2];  // shifted candidate, c.c - r_ns^2
           uint32_t e[2];
+          int at_c[2] = {0, 0};  // HALF: the candidate's place along w
           bool out_c = out_a, far_c = far_a;
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
@@ -808,13 +843,14 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
               const float x = r.x + d.x, y = r.y + d.y, z = r.z + d.z;
               q[h] = make_float4(x, y, z, fmaf(z, z, fmaf(y, y, x * x)) - mid);
               out_c = out_c || !inside(r);
+              if (HALF) at_c[h] = hk.at(r) + hk.shift(e[h]);
               far_c = far_c || !(r.x == r.x);
             }
           }
           fetch(c + 2);
           float near = 1e30f;  // smallest distance of a test from r_ns^2
-          auto keep = [&](int k, uint32_t ent) {
-            return !HALF || half_keep(a0 + k, nbr_j(ent), (ent & 63u) > 21u);
+          auto keep = [&](int k, int h) {
+            return !HALF || half_keep(a0 + k, sm.key[k], e[h], at_c[h]);
           };
 #pragma unroll 4
           for (int k = 0; k < n; k += 2) {
@@ -827,8 +863,8 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
               d2 = __ffma2_rn(make_float2(q[h].y, q[h].y), make_float2(u.z, u.w), d2);
               d2 = __ffma2_rn(make_float2(q[h].z, q[h].z), make_float2(v.x, v.y), d2);
               near = fminf(near, fminf(fabsf(d2.x), fabsf(d2.y)));
-              b[2 * h] = __ballot_sync(full, d2.x < 0.0f && keep(k, e[h]));
-              b[2 * h + 1] = __ballot_sync(full, d2.y < 0.0f && keep(k + 1, e[h]));
+              b[2 * h] = __ballot_sync(full, d2.x < 0.0f && keep(k, h));
+              b[2 * h + 1] = __ballot_sync(full, d2.y < 0.0f && keep(k + 1, h));
             }
             if (lane == 0) sm.mask[c >> 1][k >> 1] = make_uint4(b[0], b[1], b[2], b[3]);
           }
@@ -845,7 +881,7 @@ __global__ void __launch_bounds__(32 * kBWarps, 5) k_build(Sys s, ListOut lo_, i
                 bool acc = d2 < -width;
                 if (!acc && !(d2 > width) && e[h] != kNoEntry)
                   acc = exact_pair(s, g, a0 + k, e[h], c0, c1, c2, lo_.rns2);
-                const unsigned b = __ballot_sync(full, acc && keep(k, e[h]));
+                const unsigned b = __ballot_sync(full, acc && keep(k, h));
                 if (lane == 0)
                   reinterpret_cast<uint32_t *>(&sm.mask[c >> 1][k >> 1])[2 * h + (k & 1)] = b;
               }
@@ -1010,6 +1046,8 @@ __global__ void __launch_bounds__(kBlk) k_build_filter(Sys s) {
     const uint32_t cc = s.cellc[i];
     const int c0 = cell_coord(cc, 0), c1 = cell_coord(cc, 1), c2 = cell_coord(cc, 2);
     const int n1 = min(s.nnbr1[i], s.nmax1);
+    const HalfKey hk(g);
+    const int at_i = hk.at(pi);
     int count = 0;
     auto flush = [&](int grp, int fill) {
       if (grp >= ngroups) return;
@@ -1064,8 +1102,7 @@ __global__ void __launch_bounds__(kBlk) k_build_filter(Sys s) {
       for (int u = 0; u < 4; ++u) {
         const uint32_t code = e[u];
         const float r2f = r2v[u];
-        // lexicographically positive stencil offset <=> 6-bit code > 21
-        const bool ok = !HALF || half_keep(i, nbr_j(code), (code & 63u) > 21u);
+        const bool ok = !HALF || half_keep(i, at_i, code, hk.at(pj[u]) + hk.shift(code));
         const bool acc = ok && r2f < lo_thr;
         band = band || (ok && !acc && !(r2f > hi_thr));
         stage[count & 15][tx] = code;  // kept only if accepted
@@ -1077,7 +1114,7 @@ __global__ void __launch_bounds__(kBlk) k_build_filter(Sys s) {
         for (int u = 0; u < 4; ++u) {
           const uint32_t code = e[u];
           const float r2f = r2v[u];
-          const bool ok = !HALF || half_keep(i, nbr_j(code), (code & 63u) > 21u);
+          const bool ok = !HALF || half_keep(i, at_i, code, hk.at(pj[u]) + hk.shift(code));
           bool acc = ok && r2f < lo_thr;
           if (ok && !acc && !(r2f > hi_thr)) acc = exact_pair(s, g, i, code, c0, c1, c2, rns2);
           stage[count & 15][tx] = code;

@@ -18,6 +18,11 @@
 // polynomial coefficients come through L1 as in the full-list passes.  Mixed
 // path: 64-bit fixed-point accumulators (order-
 // independent, reproducible); FP64 path: FP64 reduction atomics.
+//
+// What binds the FP64 passes is the FP64 pipe.  256,000 aluminium atoms,
+// k_rho_half and k_eam_half: 650 and 898 us, 299 and 522 with polynomial
+// coefficients per interval and a floor by a rounded FMA, 283 and 490 with
+// half lists of equal length.
 #include "k_pair.cuh"
 
 namespace mdk {
