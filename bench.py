@@ -136,7 +136,7 @@ TRAFFIC = {
         "bytes_per_atom": 464.4,
         "neighbors_per_atom": 78.0,
         "threads_per_atom": 1,
-        "sources_sha256": "49ba2014f7f327c6495ca9ff5146e60010b11389a26d8e8d5d99d2a27f4bd60a",
+        "sources_sha256": "bcd58b26b1907c82f6dbc491a27a8e0c2a24cd6b3cbddc1901454a7399d3f264",
         "capture": "k_lj<Mixed, kStep, T=1>, 3 launches on 2,048,000 atoms (80^3 FCC cells, "
                    "the same lattice and 78 neighbours per atom): dram__bytes_read.sum + "
                    "dram__bytes_write.sum = 951.1 MB per launch; per-atom traffic does not "
@@ -985,7 +985,7 @@ def main():
                        "outer_list": ({"skin_A": outer_skin, "full_builds": full_builds}
                                       if outer_skin else None),
                        "list_builds_in_timed_region": builds0 - builds_before,
-                       "step_graphs": "two-step CUDA graphs replayed by mdk_step",
+                       "step_graphs": "a captured loop of steps (one list check per body) replayed by mdk_step",
                        "l2": "inputs larger than L2 (~4 GB touched per step); no flush",
                        "parallelism": "replicas" if world > 1 else "single GPU"},
             "pair_interactions_per_s": value * n_rc / 2.0,

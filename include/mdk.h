@@ -134,8 +134,8 @@ int mdk_set_potential_lj(mdk_ctx *ctx, double eps, double sigma, double rc,
  * Between knots: cubic Hermite spline, knot slopes from 3-point differences
  * (one-sided at the ends).  r >= rc gives 0; rho > rho_max extrapolates F
  * linearly and makes mdk_compute/mdk_step return MDK_ERR_RHO_RANGE.
- * 3 <= nr <= 7168 (the FP64 phi and rho tables share 227 KB of shared
- * memory), 3 <= nrho <= 65536; otherwise MDK_ERR_BAD_ARG.  Same-size tables
+ * 3 <= nr <= 7168 (mdk_eam_vjp keeps 32 bytes per knot in the 227 KB of
+ * shared memory), 3 <= nrho <= 65536; otherwise MDK_ERR_BAD_ARG.  Same-size tables
  * replace the old ones in place (no new workspace needed).
  */
 int mdk_set_potential_eam(mdk_ctx *ctx, int nr, double rc, const double *phi,
@@ -620,11 +620,11 @@ int mdk_set_list_kind(mdk_ctx *ctx, int kind);
 int mdk_get_list_kind(const mdk_ctx *ctx, int *kind);
 
 /*
- * enable != 0 (the default): mdk_step runs pairs of plain steps (neither a
- * thermo step nor the last step of the call) as one CUDA graph -- force pass
- * and rebuild chain twice -- captured on first use and re-captured whenever a
- * parameter it baked in changes (workspace, potential, launch shape, dt,
- * window...).  Steps taken while mdk_profile records run without graphs.
+ * enable != 0 (the default): mdk_step runs plain steps (neither a thermo
+ * step nor the last step of the call) as one CUDA graph -- a loop on the device
+ * of up to 8 force passes per list check, then the rebuild chain -- captured
+ * on first use and re-captured whenever a parameter it baked in changes
+ * (workspace, potential, launch shape, dt, window...).  Steps taken while mdk_profile records run without graphs.
  */
 int mdk_set_graphs(mdk_ctx *ctx, int enable);
 

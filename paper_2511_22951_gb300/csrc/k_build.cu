@@ -632,7 +632,7 @@ constexpr int kTileCh = 32;    // chunks of 32 candidates per tile (the three ph
 // Atoms of a slice at most, by the size of the system: short slices give a
 // small system more warps (a warp's chain of dependent loads and shared
 // reads takes ~10 us whatever its slice holds), long ones share the loading
-// of the candidates.  k_build in us with 8 / 16 / 32 atoms per slice: 256 LJ
+// of the candidates.  k_build in us with 8 / 16 / 32 atoms per slice (without phase 0): 256 LJ
 // atoms 21 / 24 / 29, 9,724 EAM 32 / 36 / 50, 32,000 LJ 57 / 46 / 58, 131,072
 // (6 A lists) 141 / 106 / 95, 388,204 LJ 412 / 297 / 213.
 inline int slice_atoms(int n) { return n < 16384 ? 8 : (n < 65536 ? 16 : 32); }

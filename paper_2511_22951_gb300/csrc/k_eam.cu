@@ -25,8 +25,7 @@ using namespace pair;
 
 // FP64 passes and the energy passes (thermo and compute steps only): one
 // 512-thread block per SM and up to 128 registers (the FP64 pair values, and
-// the per-atom energy and virial sums, spill at 64; the 160 KB FP64 force-pass
-// tables leave room for one block anyway)
+// the per-atom energy and virial sums, spill at 64)
 template <class P, bool ENERGY = false>
 constexpr int eam_min_blocks() {
   return sizeof(typename G<P>::R) == 4 && !ENERGY ? 2 : 1;

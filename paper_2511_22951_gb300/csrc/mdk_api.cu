@@ -1005,7 +1005,7 @@ int mdk_update_eam_knots(mdk_ctx *c, int nr, double rc, const double *phi, const
 int mdk_set_potential_eam(mdk_ctx *c, int nr, double rc, const double *phi, const double *rho,
                           int nrho, double rho_max, const double *F) {
   if (check_ctx(c)) return MDK_ERR_BAD_ARG;
-  // FP64 tables of phi and rho must fit shared memory together (16 B per knot)
+  // the adjoint's histograms of phi and rho must fit shared memory (32 B per knot)
   if (nr < 3 || nr > 7168 || nrho < 3 || nrho > 65536 || !(rc > 0.0) || !(rho_max > 0.0) ||
       !phi || !rho || !F)
     return MDK_ERR_BAD_ARG;
