@@ -68,34 +68,19 @@ __device__ __forceinline__ void lj_walk_packed(const Sys &s, const float4 *__res
   // ENERGY: compensated FP32 sums of the block sums (as the forces), in FP64
   // once per atom at the end
   Acc<float> ae, aw[6];
-  constexpr bool FINE = T >= kFineLanes;  // single entries instead of groups (walk)
-  constexpr int HALVES = FINE ? 1 : 2;    // blocks of four entries per turn
   uint4 na = make_uint4(0, 0, 0, 0), nb = na;
-  if (!FINE && kGroup * t < nn) {
+  if (kGroup * t < nn) {
     ld_group(row, na, nb);
   }
-  for (int k = FINE ? t : kGroup * t; k < nn; k += 4 * HALVES * T) {
-    uint32_t e[8];
-    if constexpr (FINE) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) e[u] = fine_entry<T>(s.nbr, Nc, i, nn, k + u * T);
-    } else {
-      const uint4 ga = na, gb = nb;
-      row += gstride * T;
-      if (k + kGroup * T < nn) {
-        ld_group(row, na, nb);
-      }
-      e[0] = ga.x;
-      e[1] = ga.y;
-      e[2] = ga.z;
-      e[3] = ga.w;
-      e[4] = gb.x;
-      e[5] = gb.y;
-      e[6] = gb.z;
-      e[7] = gb.w;
+  for (int k = kGroup * t; k < nn; k += kGroup * T) {
+    const uint4 ga = na, gb = nb;
+    row += gstride * T;
+    if (k + kGroup * T < nn) {
+      ld_group(row, na, nb);
     }
+    const uint32_t e[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
 #pragma unroll
-    for (int h = 0; h < HALVES; ++h) {
+    for (int h = 0; h < 2; ++h) {
       // whole groups: the slots past the list's length hold pad_entry, whose
       // record lies 1e18 A away (r^2 ~ 1e36 > rc^2)
       float4 q[4];

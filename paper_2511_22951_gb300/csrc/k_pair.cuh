@@ -386,11 +386,14 @@ __device__ __forceinline__ void h_scaled(R &hx, R &hy, R &hz) {
   hz *= R(0.0625);
 }
 
-// From 8 lanes per atom on, lanes take single entries t, t + T, ... instead of
-// groups of 8: a list of 78 entries has 10 groups, so of 32 lanes 10 had 8
-// entries each and 22 none; now every lane has 2 or 3 (8 lanes read one
-// group's sector).  256 FP64 LJ atoms with a warp each, run of 100 steps:
-// 1649 -> 1222 us.
+// From 8 lanes per atom on, FP64 lanes take single entries t, t + T, ...
+// instead of groups of 8: a list of 78 entries has 10 groups, so of 32 lanes
+// 10 had 8 entries each and 22 none; now every lane has 2 or 3 (8 lanes read
+// one group's sector).  256 FP64 LJ atoms with a warp each, run of 100 steps:
+// 1649 -> 1222 us.  The mixed walks keep whole groups at every T: their block
+// sums of four pairs and their lane sums are FP32, so the order of the entries
+// decides their last bits (forces ~1e-7, energies ~1e-9 relative), and an atom
+// whose groups fit the lanes of two shapes gets the same bits from both.
 constexpr int kFineLanes = 8;
 template <int T>
 __device__ __forceinline__ uint32_t fine_entry(const uint32_t *__restrict__ nbr, size_t Nc, int i,
@@ -399,7 +402,7 @@ __device__ __forceinline__ uint32_t fine_entry(const uint32_t *__restrict__ nbr,
 }
 
 // Walk the list of one atom with T lanes: lane t takes the groups of 8 list
-// words t, t + T, t + 2T, ...  A group comes in one 32-byte load; its
+// words t, t + T, t + 2T, ... (FP64 from kFineLanes on: single words).  A group comes in one 32-byte load; its
 // neighbour records are loaded four at a time before the four bodies run,
 // so each thread keeps several independent loads in flight.  `commit` runs
 // after every four pairs: the compensated per-atom sums take one block sum
@@ -408,7 +411,7 @@ template <int T, class Load, class Body, class Commit>
 __device__ __forceinline__ void walk(const uint32_t *__restrict__ nbr, size_t Nc, int i, int nn,
                                      int t, Load &&load, Body &&body, Commit &&commit) {
   using Rec = decltype(load(0u));
-  if constexpr (T >= kFineLanes) {
+  if constexpr (sizeof(Rec) == sizeof(dvec4) && T >= kFineLanes) {
     for (int k0 = t; k0 < nn; k0 += 4 * T) {
       uint32_t e[4];
       Rec q[4];
