@@ -579,7 +579,9 @@ int mdk_lj_compute_noalloc(const double *x, int64_t N, const double box_lo[3],
 int mdk_autotune(mdk_ctx *ctx, int reps, int *tpa, int *block, double *ms);
 
 /* Set the launch shape directly: tpa (list-walking lanes per atom) in {1, 2, 4, 8, 32}
- * (32: a warp per atom), block in {128, 256, 512}. */
+ * (32: a warp per atom), block in {128, 256, 512}.  The block is an upper bound: LJ
+ * runs at most 256 threads, and FP64 LJ with a warp per atom halves the block (down to
+ * a warp) while its grid has less than two blocks per SM. */
 int mdk_set_launch(mdk_ctx *ctx, int tpa, int block);
 
 /*

@@ -276,10 +276,7 @@ inline int nblk(long long n, int b) { return (int)((n + b - 1) / b); }
 
 template <class P, int MODE, bool EN, int SH, int T>
 void go(const Sys &s, const LJParams &p, StepArgs a, int block, cudaStream_t st) {
-  if (block > 256) block = 256;  // the kernel is compiled for <= 256 threads
-  // a warp per atom on few atoms: small blocks, so that they reach all SMs
-  // (the FP64 pipe of one SM serves all its warps)
-  while (T == 32 && block > 32 && s.N_cap * (32 * T / block) < 2 * 152 * 32) block /= 2;
+  block = lj_block(sizeof(typename G<P>::R) == 8 ? 0 : 1, s.N_cap, T, block);
   const int grid = nblk((long long)(s.N_cap > 0 ? s.N_cap : 1) * T, block);
   k_lj<P, MODE, EN, SH, T><<<grid, block, 0, st>>>(s, p, a);
 }
@@ -326,6 +323,25 @@ void by_mode(const Sys &s, const LJParams &p, Mode m, StepArgs a, const LaunchCf
 }
 
 }  // namespace
+
+// The block a full-list pass runs with.  The kernel is compiled for <= 256
+// threads.  FP64 with a warp per atom on few atoms: half that, down to a warp,
+// while there are less than two blocks per SM, so that the blocks reach all SMs
+// (one SM's FP64 pipe serves all its warps; 100 steps on 864 atoms 1610 -> 1428
+// us, on 256 atoms 1223 -> 1197).  Mixed passes are not bound by that pipe.
+int lj_block(int precision, int n_cap, int tpa, int block) {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (sms <= 0) sms = 1;
+  }
+  if (block > 256) block = 256;
+  while (precision == 0 && tpa == 32 && block > 32 && (long long)n_cap * 32 / block < 2 * sms)
+    block /= 2;
+  return block;
+}
 
 void launch_lj(const Sys &s, const LJParams &p, int precision, Mode mode, StepArgs a,
                const LaunchCfg &cfg, cudaStream_t st) {

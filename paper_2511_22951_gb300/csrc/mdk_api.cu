@@ -2024,6 +2024,10 @@ int mdk_autotune(mdk_ctx *c, int reps, int *tpa_out, int *block_out, double *ms_
   for (int a = 0; a < 5 && !r; ++a)
     for (int b = 0; b < 3; ++b) {
       if (c->pot == 1 && kBlock[b] > 256) continue;  // the LJ kernels take <= 256
+      if (c->pot == 1 && kind == 0 && b > 0 &&  // the same launch as the block before
+          lj_block(c->precision, (int)c->N_cap, kTpa[a], kBlock[b]) ==
+              lj_block(c->precision, (int)c->N_cap, kTpa[a], kBlock[b - 1]))
+        continue;
       if (c->pot == 3 && (a > 0 || b > 0)) continue;  // BPNN: one warp per atom, one shape
       if (kind >= 1 && (kTpa[a] != 1 || kBlock[b] > 256)) continue;  // <= 256 threads
       if (c->cfg.half != kind || !c->list_built) {

@@ -513,6 +513,8 @@ struct LaunchCfg {
                     // 2 = LJ from the cells, one warp per cell (no list)
 };
 
+// threads per block that launch_lj runs for a launch shape
+int lj_block(int precision, int n_cap, int tpa, int block);
 void launch_lj(const Sys &s, const LJParams &p, int precision, Mode mode, StepArgs a,
                const LaunchCfg &cfg, cudaStream_t st);
 // the per-atom pass that finishes a step from the accumulators in s.hacc
