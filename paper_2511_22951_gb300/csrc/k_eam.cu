@@ -49,12 +49,14 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P>()) k_rho(Sys s, EAMPara
     const int i = tl.atom(w);
     const bool valid = i < N;
     V pi;
+    uint32_t inf = 0;
     Vec<P> geo;
     int nn = 0;
     if (valid) {
       R hx, hy, hz;
       pi = GP::ld(pg + i);
-      GP::h(s.grid[GP::info(pi) >> 8], hx, hy, hz);
+      inf = GP::info(pi);
+      GP::h(s.grid[inf >> 8], hx, hy, hz);
       geo = Vec<P>(pi, hx, hy, hz);
       nn = min(s.nnbr[i], s.nmax);
     }
@@ -66,7 +68,7 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P>()) k_rho(Sys s, EAMPara
           R dx, dy, dz;
           geo.to(ent, pj, dx, dy, dz);
           const R r2 = r2_of(dx, dy, dz);
-          if (below(r2, rc2)) {
+          if (geo.inside(s.grid[inf >> 8], ent, pj, r2, rc2)) {
             int kk;
             R t;
             GP::knot(r2, inv_dr, kmax, kk, t);
@@ -140,7 +142,7 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P, ENERGY>()) k_eam(Sys s,
           R dx, dy, dz;
           geo.to(ent, pj, dx, dy, dz);
           const R r2 = r2_of(dx, dy, dz);
-          if (below(r2, rc2)) {
+          if (geo.inside(s.grid[inf >> 8], ent, pj, r2, rc2)) {
             int kk;
             R inv_r, t, dphi, drho, vphi = 0;
             GP::knot(r2, inv_dr, kmax, inv_r, kk, t);

@@ -59,7 +59,8 @@ __global__ void __launch_bounds__(256, 2) k_rho_half(Sys s, EAMParams ep, StepAr
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
     const V pi = GP::ld(pg + i);
     R hx, hy, hz;
-    GP::h(s.grid[GP::info(pi) >> 8], hx, hy, hz);
+    const Grid &g = s.grid[GP::info(pi) >> 8];
+    GP::h(g, hx, hy, hz);
     const Vec<P> geo(pi, hx, hy, hz);
     const int nn = min(s.nnbr[i], s.nmax);
     Q rho = 0;
@@ -69,7 +70,7 @@ __global__ void __launch_bounds__(256, 2) k_rho_half(Sys s, EAMParams ep, StepAr
           R dx, dy, dz;
           geo.to(ent, pj, dx, dy, dz);
           const R r2 = r2_of(dx, dy, dz);
-          if (below(r2, rc2)) {
+          if (geo.inside(g, ent, pj, r2, rc2)) {
             int kk;
             R t;
             GP::knot(r2, inv_dr, kmax, kk, t);
@@ -134,7 +135,8 @@ __global__ void __launch_bounds__(256, 2) k_eam_half(Sys s, EAMParams ep, StepAr
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
     const V pi = GP::ld(pg + i);
     R hx, hy, hz;
-    GP::h(s.grid[GP::info(pi) >> 8], hx, hy, hz);
+    const Grid &g = s.grid[GP::info(pi) >> 8];
+    GP::h(g, hx, hy, hz);
     const Vec<P> geo(pi, hx, hy, hz);
     const R fpi = fpa[i];
     const int nn = min(s.nnbr[i], s.nmax);
@@ -145,7 +147,7 @@ __global__ void __launch_bounds__(256, 2) k_eam_half(Sys s, EAMParams ep, StepAr
           R dx, dy, dz;
           geo.to(ent, pj, dx, dy, dz);
           const R r2 = r2_of(dx, dy, dz);
-          if (below(r2, rc2)) {
+          if (geo.inside(g, ent, pj, r2, rc2)) {
             int kk;
             R inv_r, t, dphi, drho;
             GP::knot(r2, inv_dr, kmax, inv_r, kk, t);

@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(256, lj_min_blocks<P, ENERGY, SHIFT>()) k_lj(S
           R dx, dy, dz;
           geo.to(ent, pj, dx, dy, dz);
           const R r2 = r2_of(dx, dy, dz);
-          if (below(r2, lc.rc2)) {
+          if (geo.inside(s.grid[inf >> 8], ent, pj, r2, lc.rc2)) {
             R fr, v;
             lj_pair<GP, SHIFT, ENERGY>(lc, r2, fr, v);
             bx += fr * dx;

@@ -67,7 +67,8 @@ __global__ void __launch_bounds__(256, half_min_blocks<P>(ENERGY))
   long long *acc = s.hacc;
   const V pi = GP::ld(pg + i);
   R hx, hy, hz;
-  GP::h(s.grid[GP::info(pi) >> 8], hx, hy, hz);
+  const Grid &g = s.grid[GP::info(pi) >> 8];
+  GP::h(g, hx, hy, hz);
   const Vec<P> geo(pi, hx, hy, hz);
   const int nn = min(s.nnbr[i], s.nmax);
   Q fx = 0, fy = 0, fz = 0, e = 0, w0 = 0, w1 = 0, w2 = 0, w3 = 0, w4 = 0, w5 = 0;
@@ -78,7 +79,7 @@ __global__ void __launch_bounds__(256, half_min_blocks<P>(ENERGY))
         R dx, dy, dz;
         geo.to(ent, pj, dx, dy, dz);
         const R r2 = r2_of(dx, dy, dz);
-        if (below(r2, lc.rc2)) {
+        if (geo.inside(g, ent, pj, r2, lc.rc2)) {
           R fr, v;
           lj_pair<GP, SHIFT, ENERGY>(lc, r2, fr, v);
           if (sizeof(R) == 4) bad = bad || !(fabs(fr) < fr_max);

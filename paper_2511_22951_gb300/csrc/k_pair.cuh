@@ -319,7 +319,7 @@ __device__ __forceinline__ double s_scaled(double, uint32_t e, int d) {
 // difference, then the shift by one FMA; r^2 = fma(dz, dz, fma(dy, dy, dx dx)).
 // Seen from j the vector is exactly minus the one seen from i, so both atoms
 // of a pair get the same r^2, bit for bit, and the same cutoff decision (FP32;
-// the FP64 kernels take Vec<Fp64>).
+// the FP64 kernels take Vec<Fp64>, whose inside() gives the same decisions).
 __device__ __forceinline__ float pvec(float pj, float pi, float sh, float h) {
   return __fmaf_rn(sh, h, __fsub_rn(pj, pi));
 }
@@ -337,7 +337,8 @@ __device__ __forceinline__ double r2_of(double dx, double dy, double dz) {
 // dimension, p - s h for s = -1, 0, 1: the FP64 pair vector component is
 // p_j - at(code of s), one FP64 operation; the choice is made by integer
 // selects (see rcp64).  Against (p_j - p_i) + s h the rounding of p - s h takes
-// the place of the difference's.
+// the place of the difference's, so seen from j the vector is minus the one seen
+// from i only to rounding (Vec<Fp64>::inside).
 struct Shift3 {
   double a, b, c;
   Shift3() = default;
@@ -364,6 +365,10 @@ struct Vec<Mixed> {
     dy = pvec(q.y, y, s_scaled(0.0f, ent, 1), hy);
     dz = pvec(q.z, z, s_scaled(0.0f, ent, 2), hz);
   }
+  __device__ __forceinline__ bool inside(const Grid &, uint32_t, const float4 &, float r2,
+                                         float rc2) const {
+    return r2 < rc2;
+  }
 };
 template <>
 struct Vec<Fp64> {
@@ -376,6 +381,19 @@ struct Vec<Fp64> {
     dx = q.x - x.at(ent);
     dy = q.y - y.at(ent >> 2);
     dz = q.z - z.at(ent >> 4);
+  }
+  // r^2 < rc^2, decided alike from both atoms of a pair and by every kernel: a
+  // pair whose r^2 lies within 2^-20 of rc^2 (high words at most 1 apart; the
+  // rounding of p - s h moves r^2 by less while |p| + h < 2^28 rc) is decided on
+  // (p_j - p_i) + s h, whose mirror image is exact.  A shell of an ideal lattice
+  // at rc would act on one atom of a pair only otherwise.
+  __device__ __forceinline__ bool inside(const Grid &g, uint32_t ent, const dvec4 &q, double r2,
+                                         double rc2) const {
+    if ((unsigned)(__double2hiint(r2) - __double2hiint(rc2) + 1) > 2u) return below(r2, rc2);
+    const double dx = __fma_rn((double)nbr_s(ent, 0), g.h[0], __dsub_rn(q.x, x.b));
+    const double dy = __fma_rn((double)nbr_s(ent, 1), g.h[1], __dsub_rn(q.y, y.b));
+    const double dz = __fma_rn((double)nbr_s(ent, 2), g.h[2], __dsub_rn(q.z, z.b));
+    return r2_of(dx, dy, dz) < rc2;
   }
 };
 

@@ -241,7 +241,9 @@ struct NaWarp {
 };
 
 // The force kernel's variant: 27-cell stencil, each stencil position one
-// periodic image, d = (x_j - x_i) + n L, pairs with r^2 < rc^2, FP64.
+// periodic image, d = x_j - (x_i - n L), pairs with r^2 < rc^2, FP64; decided on
+// (x_j - x_i) + n L, whose mirror image is exact, within 2^-20 of rc^2 (see
+// Vec<Fp64>::inside).
 // One warp per slice of a cell's atoms.  Lanes hold candidates (the 27 cells
 // flattened) and an FP32 test on cell-centre offsets drops those clearly
 // outside rc (~85%): GB300's FP64 pipe (2 lanes per clock and SM) is what
@@ -384,7 +386,15 @@ __global__ void __launch_bounds__(32 * kFWarps) k_na_force(NaParams p, unsigned 
         const double dy = s.x[kMaxAtoms + j] - gy.at(im >> 2);
         const double dz = s.x[2 * kMaxAtoms + j] - gz.at(im >> 4);
         const double r2 = r2_of(dx, dy, dz);
-        const bool in = below(r2, p.lj.rc2);
+        bool in = below(r2, p.lj.rc2);
+        if ((unsigned)(__double2hiint(r2) - __double2hiint(p.lj.rc2) + 1) <= 2u) {
+          const double ex = __fma_rn((double)nbr_s(im, 0), p.L[0], __dsub_rn(s.x[j], gx.b));
+          const double ey =
+              __fma_rn((double)nbr_s(im, 1), p.L[1], __dsub_rn(s.x[kMaxAtoms + j], gy.b));
+          const double ez =
+              __fma_rn((double)nbr_s(im, 2), p.L[2], __dsub_rn(s.x[2 * kMaxAtoms + j], gz.b));
+          in = r2_of(ex, ey, ez) < p.lj.rc2;
+        }
         double fr, u;
         lj_pair<G<Fp64>, SHIFT, true>(p.lj, r2, fr, u);
         fr = in ? fr : 0.0;
