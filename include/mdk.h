@@ -301,7 +301,8 @@ int mdk_get_neighbors(mdk_ctx *ctx, int64_t *offsets, int32_t *j, int32_t *image
  * r_ij (x) f_ij with r_ij = r_i - r_j; pressure P = (sum m v v + W)/V) at the
  * current positions.  Any output may be NULL.  f_i = sum_j V'(r_ij) r_ji/r_ji
  * (Sec. "Potentials support").  Rebuilds the lists first if needed.
- * on_device: 0 = host outputs (synchronises), 1 = device outputs.
+ * on_device: 0 = host outputs (synchronises), 1 = device outputs (E and virial: any address
+ * that a device copy reaches; F: memory that kernels of this device can write).
  */
 int mdk_compute(mdk_ctx *ctx, double *E, double *F, double *virial, int on_device);
 

@@ -713,6 +713,20 @@ uint64_t fnv(uint64_t h, const void *p, size_t n) {
   return h;
 }
 
+// Whether a kernel on the current device may store doubles at p: aligned memory
+// of this device.  Anything else that a copy can reach (an odd address, another
+// GPU's memory, host memory) is written by copies.
+bool kernel_writable(const double *p) {
+  if (!p || (reinterpret_cast<uintptr_t>(p) & 7u)) return false;
+  cudaPointerAttributes at;
+  int dev = -1;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
 uint64_t graph_key(const mdk_ctx *c, double dt) {
   uint64_t h = 1469598103934665603ull;
   h = fnv(h, &c->sys, sizeof(Sys));
@@ -1674,7 +1688,9 @@ int mdk_compute(mdk_ctx *c, double *E, double *F, double *virial, int on_device)
   Sys &s = c->sys;
   r = force_pass(c, kForceOnly, 1, 0.0);
   if (r) return r;
-  c->launches += launch_reduce(s, 0, on_device ? E : nullptr, on_device ? virial : nullptr, c->stream);
+  // the sums' kernel hands E and W out where it can store them
+  const bool E_direct = on_device && kernel_writable(E), W_direct = on_device && kernel_writable(virial);
+  c->launches += launch_reduce(s, 0, E_direct ? E : nullptr, W_direct ? virial : nullptr, c->stream);
   MDK_CK(cudaPeekAtLastError());
   c->forces_valid = true;
   c->per_atom_valid = true;
@@ -1688,6 +1704,14 @@ int mdk_compute(mdk_ctx *c, double *E, double *F, double *virial, int on_device)
   }
   if (on_device) {
     if (F) launch_store_forces(s, F, c->stream);
+    for (int q = 0; q < R; ++q) {
+      if (E && !E_direct)
+        MDK_CK(cudaMemcpyAsync(E + q, s.red + 9 * q + 1, sizeof(double), cudaMemcpyDeviceToDevice,
+                               c->stream));
+      if (virial && !W_direct)
+        MDK_CK(cudaMemcpyAsync(virial + 6 * q, s.red + 9 * q + 2, 6 * sizeof(double),
+                               cudaMemcpyDeviceToDevice, c->stream));
+    }
     MDK_CK(cudaPeekAtLastError());
     return MDK_OK;
   }
