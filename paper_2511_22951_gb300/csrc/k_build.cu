@@ -89,10 +89,11 @@ __global__ void k_pre(Sys s, int count_step, int use_cond, cudaGraphConditionalH
 // alone: 11.1), 21.2 -> 14.4 us on 32,000 mixed.  The next body reads the copy
 // that this one started from: after an odd e it is written again (by the
 // build, or by k_regather).
-__global__ void k_loop_head(Sys s, int places, cudaGraphConditionalHandle h,
+__global__ void k_loop_head(Sys s, int places, int kernels, cudaGraphConditionalHandle h,
                             cudaGraphConditionalHandle loop) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   DevStatus *st = s.st;
+  st->n_graph_kernels += kernels;
   const unsigned trig = st->trig;
   st->trig = 0u;
   if (st->abort) {
@@ -111,7 +112,6 @@ __global__ void k_loop_head(Sys s, int places, cudaGraphConditionalHandle h,
   st->left -= e;
   st->since_build += e;
   st->n_steps += e;  // index of the force evaluation that follows
-  st->n_bodies += 1;
   st->regather = e & 1;
   plan_build(s, 1);
   cudaGraphSetConditional(h, st->rebuild || st->regather ? 1u : 0u);
@@ -1153,13 +1153,14 @@ __global__ void __launch_bounds__(kBlk) k_build_filter(Sys s) {
 // A build that stepping triggered and whose list outgrew its capacity stops
 // the stepping (st->abort): the lists are truncated, so no force pass may use
 // them; the host regrows the workspace, carries the state over and resumes.
-__global__ void k_finish(Sys s, int from_graph) {
+// graph_kernels: kernels of the conditional body that this launch ends (else 0).
+__global__ void k_finish(Sys s, int graph_kernels) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   DevStatus *st = s.st;
+  st->n_graph_kernels += graph_kernels;
   if (st->rebuild) {
     st->rebuild = 0;
     st->n_builds += 1;
-    if (from_graph) st->n_graph_builds += 1;
     st->since_build = 0;
     if (st->step_build && st->build_ovf) st->abort = 1;
   }
@@ -1232,15 +1233,15 @@ int rebuild_chain_kernels(const Sys &s) {
   return (s.n_scan_blocks == 1 ? 9 : 11) + (s.win_on ? 4 : 0) + (s.outer_on ? 4 : 0);
 }
 
-void launch_loop_head(const Sys &s, int places, cudaGraphConditionalHandle h,
+void launch_loop_head(const Sys &s, int places, int kernels, cudaGraphConditionalHandle h,
                       cudaGraphConditionalHandle loop, cudaStream_t st) {
-  k_loop_head<<<1, 32, 0, st>>>(s, places, h, loop);
+  k_loop_head<<<1, 32, 0, st>>>(s, places, kernels, h, loop);
 }
 
 void launch_set_left(const Sys &s, int left, cudaStream_t st) { k_set_left<<<1, 32, 0, st>>>(s, left); }
 
-int launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_graph, int loop,
-                        cudaStream_t st) {
+void launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_graph, int loop,
+                         cudaStream_t st) {
   static int g_atom = 0, g_build = 0, g_cells = 0, g_filter = 0;
   if (g_atom == 0) {
     g_atom = persistent_blocks((const void *)k_bin, kBlk, 0);
@@ -1300,8 +1301,7 @@ int launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_gra
     else
       k_regather<Mixed, true><<<gN, kBlk, 0, st>>>(s, (float4 *)s.pg[target_pg]);
   }
-  k_finish<<<1, 32, 0, st>>>(s, from_graph);
-  return rebuild_chain_kernels(s) - 1 + (loop ? 1 : 0);
+  k_finish<<<1, 32, 0, st>>>(s, from_graph ? rebuild_chain_kernels(s) - 1 + (loop ? 1 : 0) : 0);
 }
 
 void launch_rebuild(const Sys &s, int target_pg, int precision, int count_step, cudaStream_t st) {

@@ -104,10 +104,7 @@ struct mdk_ctx {
   cudaGraphExec_t gexec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
   uint64_t gkey[2][2] = {{0, 0}, {0, 0}};
   cudaStream_t body_stream = nullptr;  // captures the conditional rebuild bodies
-  int64_t loop_kernels = 0;   // kernels of one loop body that run every time
-  int64_t body_kernels = 0;   // kernels of one conditional rebuild body
-  long long graph_builds0 = 0;  // device counts of in-graph builds and loop
-  long long bodies0 = 0;        // bodies at mdk_profile
+  long long graph_kernels0 = 0;  // device count of kernels inside graphs at mdk_profile
   double *ctr_dev = nullptr;     // cell-centre tables in the workspace
   std::vector<double> ctr_host;  // their values (kept until the upload completes)
   // moving window
@@ -537,7 +534,7 @@ __global__ void k_ckpt_begin(Sys s, int N) {
 }
 
 struct CkptCounters {
-  long long n_steps, n_builds, n_graph_builds, n_full_builds, n_inserted, n_deleted;
+  long long n_steps, n_builds, n_graph_kernels, n_full_builds, n_inserted, n_deleted;
   int since_build, next_id, outer_valid;
 };
 
@@ -546,7 +543,7 @@ __global__ void k_ckpt_end(Sys s, CkptCounters k) {
   DevStatus *st = s.st;
   st->n_steps = k.n_steps;
   st->n_builds = k.n_builds;
-  st->n_graph_builds = k.n_graph_builds;
+  st->n_graph_kernels = k.n_graph_kernels;
   st->n_full_builds = k.n_full_builds;
   st->n_inserted = k.n_inserted;
   st->n_deleted = k.n_deleted;
@@ -749,7 +746,8 @@ int loop_places(const mdk_ctx *c) { return c->N_cap * (int64_t)c->cfg.tpa <= (1 
 // after a loop body) decides and sets the value of an IF conditional node
 // whose body holds the rest of the chain, so steps without a rebuild run one
 // kernel, not the whole chain.
-int capture_conditional_chain(mdk_ctx *c, int places, cudaGraphConditionalHandle loop) {
+int capture_conditional_chain(mdk_ctx *c, int places, int kernels,
+                              cudaGraphConditionalHandle loop) {
   cudaStreamCaptureStatus cs;
   cudaGraph_t g = nullptr;
   const cudaGraphNode_t *deps = nullptr;
@@ -758,7 +756,7 @@ int capture_conditional_chain(mdk_ctx *c, int places, cudaGraphConditionalHandle
   cudaGraphConditionalHandle h;
   MDK_CK(cudaGraphConditionalHandleCreate(&h, g, 0, 0));
   if (places > 0)
-    launch_loop_head(c->sys, places, h, loop, c->cap_stream);
+    launch_loop_head(c->sys, places, kernels, h, loop, c->cap_stream);
   else
     launch_rebuild_head(c->sys, 1, h, c->cap_stream);
   MDK_CK(cudaPeekAtLastError());
@@ -774,8 +772,7 @@ int capture_conditional_chain(mdk_ctx *c, int places, cudaGraphConditionalHandle
   cudaGraph_t body = cp.conditional.phGraph_out[0];
   MDK_CK(cudaStreamBeginCaptureToGraph(c->body_stream, body, nullptr, nullptr, 0,
                                        cudaStreamCaptureModeThreadLocal));
-  c->body_kernels =
-      launch_rebuild_body(c->sys, c->cur, c->precision, 1, places > 0, c->body_stream);
+  launch_rebuild_body(c->sys, c->cur, c->precision, 1, places > 0, c->body_stream);
   const cudaError_t e = cudaPeekAtLastError();
   cudaGraph_t out = nullptr;
   MDK_CK(cudaStreamEndCapture(c->body_stream, &out));
@@ -825,8 +822,7 @@ int ensure_graph(mdk_ctx *c, int kind, int parity, double dt, uint64_t key) {
       r = force_pass(c, kStep, 0, dt, p);
       c->cur ^= 1;
     }
-    if (places > 0) c->loop_kernels = c->launches - keep_launches + 1;
-    if (!r) r = capture_conditional_chain(c, places, loop);
+    if (!r) r = capture_conditional_chain(c, places, (int)(c->launches - keep_launches) + 1, loop);
     c->stream = keep_stream;
     c->cur = keep_cur;
     c->prof = keep_prof;
@@ -1384,7 +1380,7 @@ struct CkptHeader {
   char magic[8];
   int32_t version, precision, n_rep, flags;
   int64_t N, steps_done;
-  int64_t n_steps, n_builds, n_graph_builds, n_full_builds, n_inserted, n_deleted;
+  int64_t n_steps, n_builds, n_graph_kernels, n_full_builds, n_inserted, n_deleted;
   int32_t since_build, next_id;
   double u_p;
   int64_t reserved[4];
@@ -1432,7 +1428,7 @@ int mdk_save_checkpoint(mdk_ctx *c, void *buf, size_t bytes) {
   h.steps_done = c->steps_done;
   h.n_steps = st.n_steps;
   h.n_builds = st.n_builds;
-  h.n_graph_builds = st.n_graph_builds;
+  h.n_graph_kernels = st.n_graph_kernels;
   h.n_full_builds = st.n_full_builds;
   h.n_inserted = st.n_inserted;
   h.n_deleted = st.n_deleted;
@@ -1560,7 +1556,7 @@ int mdk_load_checkpoint(mdk_ctx *c, const void *buf, size_t bytes) {
     if (!r) r = upload(2, none, s.f);
     if (r) return r;
   }
-  CkptCounters k{h.n_steps, h.n_builds, h.n_graph_builds, h.n_full_builds, h.n_inserted,
+  CkptCounters k{h.n_steps, h.n_builds, h.n_graph_kernels, h.n_full_builds, h.n_inserted,
                  h.n_deleted, h.since_build, h.next_id, (list && s.outer_on) ? 1 : 0};
   k_ckpt_end<<<1, 32, 0, c->stream>>>(s, k);
   MDK_CK(cudaPeekAtLastError());
@@ -2149,8 +2145,7 @@ int mdk_profile(mdk_ctx *c, int enable) {
     DevStatus st;
     int r = read_status(c, &st);
     if (r) return r;
-    c->graph_builds0 = st.n_graph_builds;
-    c->bodies0 = st.n_bodies;
+    c->graph_kernels0 = st.n_graph_kernels;
   }
   c->prof = enable != 0;
   c->ev_used = 0;
@@ -2181,10 +2176,9 @@ int mdk_get_profile(mdk_ctx *c, double *out) {
   out[1] = (double)c->ev_force.size();
   out[2] = total(c->ev_chain);
   out[3] = (double)c->ev_chain.size();
-  // kernels launched: those enqueued directly (and the graphs' heads), those of
-  // the loop bodies and those of the rebuild bodies that conditional nodes ran
-  out[4] = (double)c->launches + (double)c->loop_kernels * (double)(st.n_bodies - c->bodies0) +
-           (double)c->body_kernels * (double)(st.n_graph_builds - c->graph_builds0);
+  // kernels launched: those enqueued directly (and the heads of single chains),
+  // and those that graphs ran as often as the device found their conditions true
+  out[4] = (double)c->launches + (double)(st.n_graph_kernels - c->graph_kernels0);
   out[5] = (double)st.n_builds;
   out[6] = total(c->ev_kick);
   out[7] = (double)c->ev_kick.size();

@@ -63,8 +63,7 @@ struct DevStatus {
   unsigned bits;         // kSt* raised since the host last cleared them
   int max_nnbr;          // longest list seen at a build
   long long n_builds;
-  long long n_graph_builds;  // builds run inside a captured step's conditional node
-  long long n_bodies;        // loop bodies run
+  long long n_graph_kernels;  // kernels run by loop bodies and conditional rebuild bodies
   long long n_steps;
   int since_build;       // steps since the last build
   int next_id;           // id of the next atom a moving window appends
@@ -496,16 +495,16 @@ void launch_replay_filter(const Sys &s, int target_pg, int precision, cudaStream
 void launch_regather(const Sys &s, int target_pg, int precision, cudaStream_t st);
 // The same chain in two parts for captured steps: the head decides whether
 // to rebuild and sets the conditional node's value; the body (run by that
-// node only when the value is 1) rebuilds.  Returns the kernels of the body.
+// node only when the value is 1) rebuilds and counts its kernels (from_graph).
 void launch_rebuild_head(const Sys &s, int count_step, cudaGraphConditionalHandle h,
                          cudaStream_t st);
-// the head after a loop body of `places` steps: counts the steps done and sets
-// the loop's condition too
-void launch_loop_head(const Sys &s, int places, cudaGraphConditionalHandle h,
+// the head after a loop body of `places` steps: counts the steps done and the
+// body's `kernels` (its own too) and sets the loop's condition too
+void launch_loop_head(const Sys &s, int places, int kernels, cudaGraphConditionalHandle h,
                       cudaGraphConditionalHandle loop, cudaStream_t st);
 void launch_set_left(const Sys &s, int left, cudaStream_t st);
-int launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_graph, int loop,
-                        cudaStream_t st);
+void launch_rebuild_body(const Sys &s, int target_pg, int precision, int from_graph, int loop,
+                         cudaStream_t st);
 int rebuild_chain_kernels(const Sys &s);
 void launch_set_piston(const Sys &s, const uint8_t *flags, int64_t n_flags, cudaStream_t st);
 int scan_blocks_for(int n_cells);
