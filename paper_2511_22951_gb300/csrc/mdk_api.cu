@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <new>
 #include <vector>
@@ -103,6 +104,7 @@ struct mdk_ctx {
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t gexec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
   uint64_t gkey[2][2] = {{0, 0}, {0, 0}};
+  uint64_t chain_met[2] = {0, 0};  // keys of the chains last met (step_chain)
   cudaStream_t body_stream = nullptr;  // captures the conditional rebuild bodies
   long long graph_kernels0 = 0;  // device count of kernels inside graphs at mdk_profile
   double *ctr_dev = nullptr;     // cell-centre tables in the workspace
@@ -724,15 +726,27 @@ bool kernel_writable(const double *p) {
   return at.type == cudaMemoryTypeDevice && at.device == dev;
 }
 
-uint64_t graph_key(const mdk_ctx *c, double dt) {
+// What the rebuild chain of a step depends on: the system and the precision, but
+// not dt (Sys holds the noise amplitudes, which follow dt and which the chain
+// does not read) nor the potential.
+uint64_t chain_key(const mdk_ctx *c) {
   uint64_t h = 1469598103934665603ull;
-  h = fnv(h, &c->sys, sizeof(Sys));
+  const char *s = reinterpret_cast<const char *>(&c->sys);
+  const size_t a = offsetof(Sys, lang_sig), b = a + sizeof(c->sys.lang_sig);
+  h = fnv(h, s, a);
+  h = fnv(h, s + b, sizeof(Sys) - b);
+  h = fnv(h, &c->precision, sizeof(int));
+  return h;
+}
+// what a loop of steps depends on
+uint64_t loop_key(const mdk_ctx *c, uint64_t chain, double dt) {
+  uint64_t h = chain;
+  h = fnv(h, c->sys.lang_sig, sizeof(c->sys.lang_sig));
   h = fnv(h, &c->lj, sizeof(LJParams));
   h = fnv(h, &c->eam, sizeof(EAMParams));
   h = fnv(h, &c->cfg, sizeof(LaunchCfg));
   h = fnv(h, &c->pot, sizeof(int));
   h = fnv(h, &c->bp, sizeof(BPParams));
-  h = fnv(h, &c->precision, sizeof(int));
   h = fnv(h, &dt, sizeof(double));
   return h;
 }
@@ -853,10 +867,17 @@ bool use_graphs(mdk_ctx *c) {
   return cs == cudaStreamCaptureStatusNone;
 }
 
-// the rebuild chain after a step on its own (counted)
-int step_chain(mdk_ctx *c, bool graphs, double dt, uint64_t key) {
+// The rebuild chain after a step on its own (counted): its launches one by one
+// where it is met for the first time, as a graph from then on, so that a program
+// that steps once does not pay for capturing it.
+int step_chain(mdk_ctx *c, bool graphs, uint64_t key) {
   if (!graphs) return rebuild_chain(c, 1);
-  const int r = ensure_graph(c, 0, c->cur, dt, key);
+  const bool have = c->gexec[0][c->cur] && c->gkey[0][c->cur] == key;
+  if (!have && c->chain_met[c->cur] != key) {
+    c->chain_met[c->cur] = key;
+    return rebuild_chain(c, 1);
+  }
+  const int r = ensure_graph(c, 0, c->cur, 0.0, key);
   if (r) return r;
   MDK_CK(cudaGraphLaunch(c->gexec[0][c->cur], c->stream));
   c->launches += 1;
@@ -1821,7 +1842,8 @@ int mdk_step(mdk_ctx *c, double dt, int64_t nsteps) {
   }
   Sys &s = c->sys;
   const bool graphs = use_graphs(c);
-  const uint64_t key = graphs ? graph_key(c, dt) : 0;
+  const uint64_t ckey = graphs ? chain_key(c) : 0;
+  const uint64_t key = graphs ? loop_key(c, ckey, dt) : 0;
   if (c->pending) {
     // a restored mid-step state: its first half-kick, drift and list build
     // are done; the steps start with the pending force pass
@@ -1838,7 +1860,7 @@ int mdk_step(mdk_ctx *c, double dt, int64_t nsteps) {
     r = timed(c, c->ev_kick, 1, [&] { launch_kick_drift(s, c->precision, a, c->stream); });
     if (r) return r;
     c->cur ^= 1;
-    r = step_chain(c, graphs, dt, key);
+    r = step_chain(c, graphs, ckey);
     if (r) return r;
   }
   auto is_thermo = [&](int64_t q) {
@@ -1874,7 +1896,7 @@ int mdk_step(mdk_ctx *c, double dt, int64_t nsteps) {
     }
     if (!last) {
       c->cur ^= 1;
-      r = step_chain(c, graphs, dt, key);
+      r = step_chain(c, graphs, ckey);
       if (r) return r;
     }
   }
