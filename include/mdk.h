@@ -144,11 +144,12 @@ int mdk_set_potential_eam(mdk_ctx *ctx, int nr, double rc, const double *phi,
 
 /*
  * New knot values for the tables of mdk_set_potential_eam, from device arrays
- * on the context's stream (a fitting loop's parameters stay on the GPU: no
- * host copy, no synchronisation).  Same nr and nrho as before, with a
- * workspace set; otherwise MDK_ERR_ORDER and nothing changes (use
- * mdk_set_potential_eam).  rc and rho_max may change.  Results are those of
- * mdk_set_potential_eam with the same values.
+ * of the context's device, on its stream (a fitting loop's parameters stay on
+ * the GPU: no synchronisation; the first call allocates a pinned host copy, which
+ * every call renews asynchronously for a later workspace).  Same nr and nrho as
+ * before, with a workspace set and the stream not being captured; otherwise
+ * MDK_ERR_ORDER and nothing changes (use mdk_set_potential_eam).  rc and rho_max
+ * may change.  Results are those of mdk_set_potential_eam with the same values.
  */
 int mdk_update_eam_knots(mdk_ctx *ctx, int nr, double rc, const double *phi, const double *rho,
                          int nrho, double rho_max, const double *F);

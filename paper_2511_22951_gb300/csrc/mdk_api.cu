@@ -858,14 +858,15 @@ int ensure_graph(mdk_ctx *c, int kind, int parity, double dt, uint64_t key) {
   return MDK_OK;
 }
 
-// whether a call steps with graphs: not while profiling, and not while the
-// caller captures the stream (the steps then go into that graph one by one)
-bool use_graphs(mdk_ctx *c) {
-  if (!c->graphs_on || c->prof) return false;
+bool capturing(mdk_ctx *c) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) cudaGetLastError();
-  return cs == cudaStreamCaptureStatusNone;
+  return cs != cudaStreamCaptureStatusNone;
 }
+
+// whether a call steps with graphs: not while profiling, and not while the
+// caller captures the stream (the steps then go into that graph one by one)
+bool use_graphs(mdk_ctx *c) { return c->graphs_on && !c->prof && !capturing(c); }
 
 // The rebuild chain after a step on its own (counted): its launches one by one
 // where it is met for the first time, as a graph from then on, so that a program
@@ -1013,6 +1014,8 @@ int mdk_update_eam_knots(mdk_ctx *c, int nr, double rc, const double *phi, const
                          int nrho, double rho_max, const double *F) {
   if (check_ctx(c) || !(rc > 0.0) || !(rho_max > 0.0) || !phi || !rho || !F) return MDK_ERR_BAD_ARG;
   if (c->pot != 2 || c->eam.nr != nr || c->eam.nrho != nrho || !c->ws_ok) return MDK_ERR_ORDER;
+  // the host copy below would hold the knots only once the captured graph runs
+  if (capturing(c)) return MDK_ERR_ORDER;
   const size_t n = (size_t)2 * nr + nrho;
   if (n > c->eam_pinned_n) {
     double *p = nullptr;

@@ -230,10 +230,22 @@ class Context:
         self.version += 1
 
     def update_eam_knots(self, phi, rho, F, rc, rho_max):
-        """New knot values of the current tables from float64 CUDA tensors of
-        the same sizes, enqueued on the context's stream.  False (and nothing
-        changed) when the sizes differ or no workspace is set yet: then
-        set_potential_eam is the call."""
+        """New knot values of the current tables from contiguous float64 CUDA
+        vectors of the context's device (anything else: ValueError) of the
+        same sizes, enqueued on the context's stream.  False (and nothing
+        changed) when the sizes differ, no workspace is set yet or the stream
+        is being captured: then set_potential_eam is the call."""
+        for t in (phi, rho, F):
+            if not (t.is_cuda and t.dtype == self.torch.float64 and t.dim() == 1 and
+                    t.is_contiguous()):
+                raise ValueError("knots have to be contiguous float64 CUDA vectors")
+        dev = self.device.index
+        if dev is None:
+            dev = self.torch.cuda.current_device()
+        if any(t.device.index != dev for t in (phi, rho, F)):
+            raise ValueError("knots have to be on the context's device")
+        if rho.shape != phi.shape:
+            raise ValueError("phi and rho have to have the same number of knots")
         r = self.lib.mdk_update_eam_knots(self.h, phi.shape[0], rc, _ptr(phi), _ptr(rho),
                                           F.shape[0], rho_max, _ptr(F))
         if r == MDK_ERR_ORDER:
