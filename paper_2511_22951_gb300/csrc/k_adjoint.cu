@@ -84,19 +84,27 @@ struct Fx64 {
     if (old + vl < old) vh += 1;
     if (vh != 0) atomicAdd(hi + slot, vh);
   }
-  __device__ __forceinline__ void add(int slot, double w) const {
+  __device__ __forceinline__ void add(int slot, double w, bool) const {
     const long long v = __double2ll_rn(w);
     add(slot, (unsigned)v, (int)(v >> 32));
   }
   // A float rounded to 64 bits without the conversion to int64, which runs on
   // GB300's FP64 pipe (16 cycles of an SM per warp; 8 conversions a pair kept
-  // that pipe 89% busy): the high word by an FMA at 1.5 2^23 (|w| < 2^53, see
-  // k_adj_scale), the exact rest (at most 2^31 in magnitude) to 32 bits.
+  // that pipe 89% busy): the high word by an FMA at 1.5 2^23 (|w| < 2^53;
+  // wide: terms may be larger, see k_adj_scale), the exact rest (at most 2^31
+  // in magnitude; +2^31 itself, a tie, saturates and is put right) to 32 bits.
   // k_adj_pair on the 143,460-atom cold-curve batch 243 -> 183 us.
-  __device__ __forceinline__ void add(int slot, float w) const {
+  __device__ __forceinline__ void add(int slot, float w, bool wide) const {
+    if (wide) {
+      const long long v = __float2ll_rn(w);
+      add(slot, (unsigned)v, (int)(v >> 32));
+      return;
+    }
     const float m = fmaf(w, 0x1p-32f, 12582912.0f);
-    const int vl = __float2int_rn(fmaf(m - 12582912.0f, -0x1p32f, w));
-    add(slot, (unsigned)vl, __float_as_int(m) - 0x4B400000 + (vl >> 31));
+    const float rest = fmaf(m - 12582912.0f, -0x1p32f, w);
+    const int vl = __float2int_rn(rest);
+    add(slot, (unsigned)vl + (rest == 0x1p31f ? 1u : 0u),
+        __float_as_int(m) - 0x4B400000 + (vl >> 31));
   }
   __device__ __forceinline__ long long get(int slot) const {
     return (long long)(((unsigned long long)(unsigned)hi[slot] << 32) | lo[slot]);
@@ -106,12 +114,13 @@ struct Fx64 {
 // fixed-point add of cv * (value weights) + cd * (derivative weights) to the
 // slots (y_k, M_k, y_{k+1}, M_{k+1}) = 2k .. 2k + 3
 template <class R>
-__device__ __forceinline__ void scatter_fx(const Fx64 &h, int k, R S, R a0, R a1, R a2, R a3) {
+__device__ __forceinline__ void scatter_fx(const Fx64 &h, bool wide, int k, R S, R a0, R a1, R a2,
+                                           R a3) {
   // S is a power of two, so the products are exact
-  h.add(2 * k, a0 * S);
-  h.add(2 * k + 1, a1 * S);
-  h.add(2 * k + 2, a2 * S);
-  h.add(2 * k + 3, a3 * S);
+  h.add(2 * k, a0 * S, wide);
+  h.add(2 * k + 1, a1 * S, wide);
+  h.add(2 * k + 2, a2 * S, wide);
+  h.add(2 * k + 3, a3 * S, wide);
 }
 
 // add a block's shared histogram to the global one (zeros skipped)
@@ -272,9 +281,9 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_c(Sys s, EAMParams ep, AdjArg
 }
 
 // ---- the fixed-point scale of pass pair (one thread) ---------------------------------
-// fp32: the mixed path's terms also stay below 2^53 (Fx64::add; a limit for
-// systems of a few atoms only, where P B would allow more)
-__global__ void k_adj_scale(Sys s, EAMParams ep, AdjArgs a, int fp32) {
+// terms stay below 2^62 / P; on systems of a few atoms (P < 512) that is above
+// the 2^53 of the short conversion (Fx64::add), so aux[5] tells the pairs
+__global__ void k_adj_scale(Sys s, EAMParams ep, AdjArgs a) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const double gE = __longlong_as_double(a.aux[0]), gF = __longlong_as_double(a.aux[1]);
   const double lam = __longlong_as_double(a.aux[2]), fp = __longlong_as_double(a.aux[3]);
@@ -283,11 +292,11 @@ __global__ void k_adj_scale(Sys s, EAMParams ep, AdjArgs a, int fp32) {
   double S = 1.0;
   if (P * B > 0.0 && isfinite(P * B)) {
     int e = 61 - (int)ceil(log2(P * B));
-    if (fp32) e = min(e, 52 - (int)ceil(log2(B)));
     e = e > 100 ? 100 : (e < -100 ? -100 : e);  // a finite FP32 scale too
     S = ldexp(1.0, e);
   }
   a.aux[4] = __double_as_longlong(S);
+  a.aux[5] = B * S <= 0x1p52 ? 0 : 1;
 }
 
 // ---- pass pair: phi- and rho-knot weights of every pair -------------------------------
@@ -304,6 +313,7 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_pair(Sys s, EAMParams ep, Adj
   for (int q = threadIdx.x; q < 8 * ep.nr; q += blockDim.x) w[q] = 0u;
   __syncthreads();
   const R S = (R)__longlong_as_double(a.aux[4]);
+  const bool wide = a.aux[5] != 0;
   const int N = s.st->N;
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
@@ -352,9 +362,9 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_pair(Sys s, EAMParams ep, Adj
             const R gd = (gix * dx + giy * dy + giz * dz) * inv_r;
             const R cp = gd * inv_dr;                    // phi': (gF_i . d^) / h
             const R cr = gd * (fpi + q.fp) * inv_dr;     // rho': times F'_i + F'_j
-            scatter_fx<R>(hp, kk, S, half_gE * w[0] + cp * dw[0], half_gE * w[1] + cp * dw[1],
+            scatter_fx<R>(hp, wide, kk, S, half_gE * w[0] + cp * dw[0], half_gE * w[1] + cp * dw[1],
                           half_gE * w[2] + cp * dw[2], half_gE * w[3] + cp * dw[3]);
-            scatter_fx<R>(hr, kk, S, lam * w[0] + cr * dw[0], lam * w[1] + cr * dw[1],
+            scatter_fx<R>(hr, wide, kk, S, lam * w[0] + cr * dw[0], lam * w[1] + cr * dw[1],
                           lam * w[2] + cr * dw[2], lam * w[3] + cr * dw[3]);
           }
         },
@@ -441,7 +451,7 @@ int run(const Sys &s, const EAMParams &ep, const double *gF, AdjArgs a, int64_t 
   const int N = (int)n_atoms;
   k_adj_load<P><<<nblk(s.N_cap > 0 ? s.N_cap : 1, 256), 256, 0, st>>>(s, gF, a);
   k_adj_c<P><<<persistent_grid(k_adj_c<P>, b_c, N), kAdjBlock, b_c, st>>>(s, ep, a);
-  k_adj_scale<<<1, 32, 0, st>>>(s, ep, a, sizeof(typename GP::R) == 4);
+  k_adj_scale<<<1, 32, 0, st>>>(s, ep, a);
   k_adj_pair<P><<<persistent_grid(k_adj_pair<P>, b_p, N), kAdjBlock, b_p, st>>>(s, ep, a);
   k_adj_fin<<<nblk(2 * ep.nr + ep.nrho, 256), 256, 0, st>>>(ep, a);
   return 0;

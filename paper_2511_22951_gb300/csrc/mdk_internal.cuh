@@ -579,7 +579,7 @@ struct AdjArgs {
   longlong2 *acc_phi, *acc_rho;      // per knot: (d/dy, d/dM), fixed point (units 1/S)
   double2 *acc_F;                    // per knot: (d/dy, d/dM), FP64
   long long *aux;                    // [0..3] bounds (bits of max |gE|, |gF_i|, |lambda|,
-                                     // |F'|), [4] the fixed-point scale S (bits of a double)
+                                     // |F'|), [4] the fixed-point scale S (bits of a double), [5] 1: terms may reach 2^53
   double *out;                       // [2 nr + nrho] knot gradients (phi | rho | F)
 };
 int adjoint_smem_bytes(const EAMParams &ep, int precision, int pass);
