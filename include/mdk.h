@@ -530,7 +530,7 @@ int mdk_eam_vjp(mdk_ctx *ctx, const double *gE, const double *gF, double *dtheta
  * variant of the force kernel behind mdk_compute.)
  *
  * Its scratch (cell histogram and starts, atoms sorted by cell, wrapped
- * positions, per-atom energies: about 2.5 MB) is one file-scope __device__
+ * positions, one energy per block: 2.0 MB) is one file-scope __device__
  * array in libmdk.so, which every GPU that loads the library holds until the
  * process exits.  The first call on a device looks that array's address up
  * (with the device current) and keeps it; make the first call on each device

@@ -1027,9 +1027,10 @@ __global__ void __launch_bounds__(kBlk) k_outer_refresh(Sys s) {
   }
 }
 
-// the Verlet list (full or half) from the outer list: the same FP32
-// pre-filter, band and exact FP64 test as k_build, on the outer list's
-// candidates in their order (so the list equals a build from the cells)
+// the Verlet list (full or half) from the outer list: an FP32 pre-filter whose
+// band (filt_lo .. filt_hi) is its own, and inside it the exact FP64 test that
+// k_build ends in too, on the outer list's candidates in their order, so the
+// list equals a build from the cells
 template <bool HALF>
 __global__ void __launch_bounds__(kBlk) k_build_filter(Sys s) {
   __shared__ uint32_t stage[2 * kGroup][kBlk];
@@ -1086,7 +1087,7 @@ __global__ void __launch_bounds__(kBlk) k_build_filter(Sys s) {
       const float2 dz = __ffma2_rn(sz, hz2, __fadd2_rn(make_float2(qa.z, qb.z), mpz));
       return __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
     };
-    // four candidates at a time (as k_build's blocks of four)
+    // four candidates at a time: their gathers go out together
     auto block4 = [&](const uint32_t *e) {
       const int before = count;
       // whole groups: slots past n1 hold pad_entry, whose record (pf[N_cap])

@@ -61,8 +61,8 @@ constexpr int kRedThreads = 256;
 
 // The block's sums of acc[0..7]; thread c < 8 gets the sum of value c.  Three
 // exchanges halve the values that a lane carries while they double the lanes
-// that are summed (lane l ends with value (l >> 2) & 7 in bit-reversed order),
-// two more finish the warp; then warps in order.
+// that are summed (lane l ends with value l >> 2), two more finish the warp;
+// then warps in order.
 __device__ __forceinline__ double block_sum8(double (&acc)[8]) {
   __shared__ double sh[8][kRedThreads / 32];
   const unsigned full = 0xffffffffu;

@@ -59,7 +59,8 @@ constexpr size_t kOffCell = kOffAtom + 4 * (size_t)kMaxAtoms;
 constexpr size_t kOffX = kOffCell + 4 * (size_t)kMaxAtoms;
 constexpr size_t kOffP = kOffX + 24 * (size_t)kMaxAtoms;
 constexpr size_t kOffE = kOffP + 16 * (size_t)kMaxAtoms;
-constexpr size_t kOffMisc = kOffE + 8 * (size_t)kMaxAtoms;
+constexpr size_t kMaxBlocks = kMaxAtoms / (kSlice * kFWarps);  // of the force kernel
+constexpr size_t kOffMisc = kOffE + 8 * kMaxBlocks;
 constexpr size_t kScratchBytes = kOffMisc + 256;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
