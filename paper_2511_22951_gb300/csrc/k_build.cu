@@ -632,10 +632,13 @@ constexpr int kTileCh = 32;    // chunks of 32 candidates per tile (the three ph
 // Atoms of a slice at most, by the size of the system: short slices give a
 // small system more warps (a warp's chain of dependent loads and shared
 // reads takes ~10 us whatever its slice holds), long ones share the loading
-// of the candidates.  k_build in us with 8 / 16 / 32 atoms per slice (without phase 0): 256 LJ
-// atoms 21 / 24 / 29, 9,724 EAM 32 / 36 / 50, 32,000 LJ 57 / 46 / 58, 131,072
-// (6 A lists) 141 / 106 / 95, 388,204 LJ 412 / 297 / 213.
-inline int slice_atoms(int n) { return n < 16384 ? 8 : (n < 65536 ? 16 : 32); }
+// of the candidates.  The steps lie where the slices of one size no longer fit one
+// round of blocks.  k_build in us with 8 / 16 / 32 atoms per slice: 9,724 EAM atoms
+// 29 / 31 / 44, 13,500 EAM 29 / 35 / 47, 19,652 EAM 34 / 36 / 47 and LJ 36 / 35 / 48,
+// 32,000 EAM 52 / 36 / 49 and LJ 53 / 41 / 44, 42,592 EAM 58 / 40 / 49 and LJ 65 /
+// 43 / 52, 50,688 LJ 70 / 56 / 53, 55,296 EAM 73 / 62 / 53, 62,500 LJ 85 / 73 / 58,
+// 131,072 (6 A lists) 137 / 100 / 90, 388,204 LJ 405 / 290 / 201.
+inline int slice_atoms(int n) { return n < 24576 ? 8 : (n < 49152 ? 16 : 32); }
 struct BuildWarp {
   uint32_t ent[kTileCh * 32];      // list entries of the tile's candidates, by chunk and lane
   uint4 mask[kTileCh / 2][16];     // per chunk and atom pair: (c, k), (c, k+1), (c+1, k), (c+1, k+1)
