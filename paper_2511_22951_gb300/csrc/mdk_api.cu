@@ -753,8 +753,12 @@ uint64_t loop_key(const mdk_ctx *c, uint64_t chain, double dt) {
 
 // Steps that one loop body holds.  A place after a triggered build does
 // nothing, but its blocks still start and exit (~1 us for a small grid, ~60 us
-// for 65,000 blocks), and a build comes about every ten steps.
-int loop_places(const mdk_ctx *c) { return c->N_cap * (int64_t)c->cfg.tpa <= (1 << 22) ? 8 : 2; }
+// for 65,000 blocks), and a build comes about every ten steps.  LJ argon mixed,
+// 41 steps with 3 to 4 builds, us a step with 8 / 2 places: 32,000 atoms (two lanes
+// each) 18.4 / 20.1, 388,204 atoms (one lane, as below) 83.0 / 84.8, 1,048,576 204.6 /
+// 205.6, 2,048,000 381.9 / 378.3, 3,538,944 583.7 / 580.6, 8,388,608 1313.8 / 1299.5;
+// 4 places lie between or within 0.2% of the better.
+int loop_places(const mdk_ctx *c) { return c->N_cap * (int64_t)c->cfg.tpa <= (3 << 19) ? 8 : 2; }
 
 // The rebuild chain of captured steps: the head kernel (k_pre, or k_loop_head
 // after a loop body) decides and sets the value of an IF conditional node

@@ -110,6 +110,6 @@ def test_overflow_inside_a_body(mdk, prec, kind):
     ((2, 3, 4, 5), 0, 0.0, False), ((18, 7), 0, 0.0, True), ((11, 12), 3, 0.0, False),
     ((9, 8), 1, 0.0, False), ((21, 10), 0, 1.5, False), ((12, 9), 2, 1.5, True)])
 def test_two_places(mdk, runs, every, outer, lang):
-    """143,748 atoms, a warp per atom: more than 2^22 lanes."""
+    """143,748 atoms, a warp per atom: 4.6 million lanes."""
     check(mdk, pot="lj", prec="mixed", kind="full", runs=runs, every=every, outer=outer, lang=lang,
           cells=(33, 33, 33), tpa=32)
