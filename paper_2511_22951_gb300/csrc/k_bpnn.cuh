@@ -248,20 +248,20 @@ __device__ __forceinline__ R sep2(const Q4<R> &a, const Q4<R> &b) {
   return sx * sx + sy * sy + sz * sz;
 }
 // e^x of both components: 2^(x log2 e), results below the normal range flushed
-__device__ __forceinline__ P2<float> ex2(P2<float> x) {
+__device__ __forceinline__ P2<float> exp_both(P2<float> x) {
   const P2<float> y = mul2(x, both(1.4426950408889634f));
   P2<float> r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(y.x));
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(y.y));
   return r;
 }
-__device__ __forceinline__ P2<double> ex2(P2<double> x) { return {exp(x.x), exp(x.y)}; }
+__device__ __forceinline__ P2<double> exp_both(P2<double> x) { return {exp(x.x), exp(x.y)}; }
 // exp(-eta R_ab^2) of (eta, kind) groups p and p + 1 (K4 false: of those of kind 4)
 template <bool K4, class R>
 __device__ __forceinline__ P2<R> gauss2(const BPParams &bp, int p, R rab2) {
   const bool k0 = K4 || bp.y_kind[p] == 4, k1 = K4 || bp.y_kind[p + 1] == 4;
   if (k0 && k1)
-    return ex2(mul2({pick<R>(bp.y_meta[p], bp.y_metaf[p]),
+    return exp_both(mul2({pick<R>(bp.y_meta[p], bp.y_metaf[p]),
                      pick<R>(bp.y_meta[p + 1], bp.y_metaf[p + 1])}, both(rab2)));
   P2<R> r = both(R(0));
   if (k0) r.x = BM<R>::ex(pick<R>(bp.y_meta[p], bp.y_metaf[p]) * rab2);

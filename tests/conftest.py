@@ -18,3 +18,14 @@ def ora():
     import oracle
     oracle.build()
     return oracle
+
+
+@pytest.fixture(scope="session")
+def mdk():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2511_22951_gb300 import _build, mdk as m
+    _build.build()
+    m.load()
+    return m

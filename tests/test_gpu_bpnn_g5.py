@@ -12,17 +12,6 @@ from paper_2511_22951_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def mdk():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2511_22951_gb300 import _build, mdk as m
-    _build.build()
-    m.load()
-    return m
-
-
 def model(groups, kinds, rc=5.0):
     """groups (eta, kind) groups of 8 functions; kinds: 5, 4 or 45 (in turn)."""
     m = W.maise_like_bpnn(0, rc=rc, n_ang=8)

@@ -17,17 +17,6 @@ from test_gpu_parity import eam_ctx, lj_ctx
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def mdk():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2511_22951_gb300 import _build, mdk as m
-    _build.build()
-    m.load()
-    return m
-
-
 # lattice constant, shell (rc = a sqrt(shell / 2)), offset of the lattice
 CASES = [(5.26, 4, 0.3), (5.13, 5, 1.7), (5.4, 4, 0.11)]
 NEIGH = 100          # more than the neighbours of the fifth shell

@@ -13,17 +13,6 @@ from paper_2511_22951_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def mdk():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2511_22951_gb300 import _build, mdk as m
-    _build.build()
-    m.load()
-    return m
-
-
 def by_hand(n, every):
     since, total = 1, 1 + 1                 # kick, check
     if every and since >= every:

@@ -13,17 +13,6 @@ from test_gpu_parity import eam_ctx
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def mdk():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2511_22951_gb300 import _build, mdk as m
-    _build.build()
-    m.load()
-    return m
-
-
 def system():
     rng = np.random.default_rng(2)
     x = W.fcc_lattice(4, 4, 5, 3.6) + rng.normal(0, 0.05, (320, 3))

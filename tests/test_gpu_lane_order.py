@@ -13,17 +13,6 @@ from test_gpu_parity import eam_ctx, lj_ctx
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def mdk():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2511_22951_gb300 import _build, mdk as m
-    _build.build()
-    m.load()
-    return m
-
-
 # spacing over the cutoff, share of the sites taken, most entries: 12, 18 and
 # 42 neighbours of the full lattice
 LATTICES = [(1.35, 0.3, 8), (1.35, 1.0, 16), (0.95, 1.0, 32), (0.79, 1.0, 64)]

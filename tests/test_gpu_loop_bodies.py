@@ -13,17 +13,6 @@ from paper_2511_22951_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def mdk():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2511_22951_gb300 import _build, mdk as m
-    _build.build()
-    m.load()
-    return m
-
-
 POTS = {  # potential: (lattice constant, mass, T, dt)
     "lj": (5.3, W.MASS_AR, 400.0, 3.0),
     "eam": (4.05, W.MASS_AL, 900.0, 2.0),

@@ -15,12 +15,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("cells,take", [((16, 32, 16), 32768), ((4, 4, 4), 16), ((4, 4, 4), 17), ((4, 4, 4), 1)])
-def test_sizes(cells, take):
+def test_sizes(mdk, cells, take):
     import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2511_22951_gb300 import _build, mdk
-    _build.build()
     rng = np.random.default_rng(2)
     a, lj = 5.26, W.LJ_AR
     x = W.fcc_lattice(*cells, a)[:take] + rng.normal(0, 0.05, (take, 3))

@@ -14,17 +14,6 @@ pytestmark = pytest.mark.gpu
 P = ctypes.c_void_p
 
 
-@pytest.fixture(scope="module")
-def mdk():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2511_22951_gb300 import _build, mdk as m
-    _build.build()
-    m.load()
-    return m
-
-
 def place(torch, where, n):
     """(address, reader) of n doubles."""
     if where == "pinned":

@@ -16,17 +16,6 @@ from paper_2511_22951_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def mdk():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2511_22951_gb300 import _build, mdk as m
-    _build.build()
-    m.load()
-    return m
-
-
 def context(mdk, lang):
     rng = np.random.default_rng(1)
     s = W.lattice_system(rng, (5, 5, 5), 5.26, W.MASS_AR, 20.0, sigma_jitter=0.02)
