@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P, ENERGY>()) k_eam(Sys s,
     tab = GP::pr8(ep);  // one 32-byte record per interval
   else
     tab = GP::pr(ep);
-  const int N = run_n(s, a);
+  const int N = run_n<MODE>(s, a);
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
   const V *__restrict__ pgf = (const V *)s.pgF;  // neighbours: offsets and F'
@@ -117,15 +117,17 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P, ENERGY>()) k_eam(Sys s,
     const bool valid = i < N;
     V pi;
     uint32_t inf = 0;
-    R fpi = 0;
-    Vec<P> geo;
+    R hx = 0, hy = 0, hz = 0, fpi = 0;
+    Vec<P> geo;  // FP64
     int nn = 0;
     if (valid) {
-      R hx, hy, hz;
       pi = GP::ld(pg + i);
       inf = GP::info(pi);
       GP::h(s.grid[inf >> 8], hx, hy, hz);
-      geo = Vec<P>(pi, hx, hy, hz);
+      if constexpr (sizeof(R) == 4)
+        h_scaled(hx, hy, hz);  // for s_scaled
+      else
+        geo = Vec<P>(pi, hx, hy, hz);
       fpi = __ldcs(fpa + i);
       nn = min(s.nnbr[i], s.nmax);
     }
@@ -140,7 +142,13 @@ __global__ void __launch_bounds__(512, eam_min_blocks<P, ENERGY>()) k_eam(Sys s,
         s.nbr, Nc, i, nn, tl.t, [&](uint32_t j) { return GP::ld(pgf + dbg_idx(s, j, Nc)); },
         [&](uint32_t ent, const V &pj) {
           R dx, dy, dz;
-          geo.to(ent, pj, dx, dy, dz);
+          if constexpr (sizeof(R) == 4) {  // as Vec<Mixed>, on pi and h (256,000 atoms 71.6 -> 70.6 us)
+            dx = pvec((R)pj.x, (R)pi.x, s_scaled(R(0), ent, 0), hx);
+            dy = pvec((R)pj.y, (R)pi.y, s_scaled(R(0), ent, 1), hy);
+            dz = pvec((R)pj.z, (R)pi.z, s_scaled(R(0), ent, 2), hz);
+          } else {
+            geo.to(ent, pj, dx, dy, dz);
+          }
           const R r2 = r2_of(dx, dy, dz);
           if (geo.inside(s.grid[inf >> 8], ent, pj, r2, rc2)) {
             int kk;

@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(256, lj_min_blocks<P, ENERGY, SHIFT>()) k_lj(S
   using GP = G<P>;
   using R = typename GP::R;
   using V = typename GP::V;
-  const int N = run_n(s, a);
+  const int N = run_n<MODE>(s, a);
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
   const LJc<R> lc(lp);

@@ -476,6 +476,13 @@ __device__ __forceinline__ int run_n(const Sys &s, const StepArgs &a) {
   }
   return wait ? 0 : N;
 }
+// the same where MODE is known: force-only passes are never part of a loop body
+// (and their code, which the autotuner times, holds nothing of the loop)
+template <int MODE>
+__device__ __forceinline__ int run_n(const Sys &s, const StepArgs &a) {
+  if (MODE == kForceOnly) return s.st->abort ? 0 : s.st->N;
+  return run_n(s, a);
+}
 // an atom moved past skin/2: the lists are rebuilt before the next step
 __device__ __forceinline__ void trigger_build(const Sys &s, const StepArgs &a) {
   if (a.pos < 0)
