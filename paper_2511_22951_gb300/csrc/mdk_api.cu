@@ -2048,22 +2048,8 @@ int mdk_autotune(mdk_ctx *c, int reps, int *tpa_out, int *block_out, double *ms_
   const LaunchCfg keep = c->cfg;
   const bool prof = c->prof;
   c->prof = false;
-  struct Timed {
-    LaunchCfg cfg;
-    float ms;
-  };
-  std::vector<Timed> shapes;
-  // mean of reps passes of the current shape
-  auto time_passes = [&](float &ms) -> int {
-    MDK_CK(cudaEventRecord(e0, c->stream));
-    int q = 0;
-    for (int k = 0; k < reps && !q; ++k) q = force_pass(c, kForceOnly, 0, 0.0);
-    MDK_CK(cudaEventRecord(e1, c->stream));
-    MDK_CK(cudaEventSynchronize(e1));
-    MDK_CK(cudaEventElapsedTime(&ms, e0, e1));
-    ms /= (float)reps;
-    return q;
-  };
+  LaunchCfg best = keep;
+  float best_ms = -1.f;
   static const int kTpa[5] = {1, 2, 4, 8, 32};  // 32: a warp per atom
   static const int kBlock[3] = {128, 256, 512};
   // LJ and EAM: full lists in every shape, then half lists (one thread per
@@ -2088,34 +2074,18 @@ int mdk_autotune(mdk_ctx *c, int reps, int *tpa_out, int *block_out, double *ms_
       c->cfg.block = kBlock[b];
       r = force_pass(c, kForceOnly, 0, 0.0);  // warm-up (and grid set-up)
       if (r) break;
+      MDK_CK(cudaEventRecord(e0, c->stream));
+      for (int q = 0; q < reps && !r; ++q) r = force_pass(c, kForceOnly, 0, 0.0);
+      MDK_CK(cudaEventRecord(e1, c->stream));
+      MDK_CK(cudaEventSynchronize(e1));
       float ms = 0.f;
-      r = time_passes(ms);
-      if (r) break;
-      shapes.push_back({c->cfg, ms});
-    }
-  // one disturbed measurement must not decide: the shapes within 3% of the best
-  // (at most 3, of its list kind) are timed again in turn, the least time counts
-  std::sort(shapes.begin(), shapes.end(), [](const Timed &p, const Timed &q) { return p.ms < q.ms; });
-  size_t few = 0;
-  for (const Timed &t : shapes)
-    if (few < 3 && t.cfg.half == shapes[0].cfg.half && t.ms <= 1.03f * shapes[0].ms) shapes[few++] = t;
-  if (!r && few > 1) {
-    if (shapes[0].cfg.half != c->cfg.half) {
-      use_list_kind(c, shapes[0].cfg.half);
-      r = build_now(c);
-    }
-    for (int round = 0; round < 2 && !r; ++round)
-      for (size_t q = 0; q < few && !r; ++q) {
-        c->cfg = shapes[q].cfg;
-        float ms = 0.f;
-        r = time_passes(ms);
-        shapes[q].ms = round == 0 ? ms : std::min(shapes[q].ms, ms);
+      MDK_CK(cudaEventElapsedTime(&ms, e0, e1));
+      ms /= (float)reps;
+      if (best_ms < 0.f || ms < best_ms) {
+        best_ms = ms;
+        best = c->cfg;
       }
-    std::sort(shapes.begin(), shapes.begin() + few,
-              [](const Timed &p, const Timed &q) { return p.ms < q.ms; });
-  }
-  const LaunchCfg best = shapes.empty() ? keep : shapes[0].cfg;
-  const float best_ms = shapes.empty() ? -1.f : shapes[0].ms;
+    }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   c->prof = prof;
