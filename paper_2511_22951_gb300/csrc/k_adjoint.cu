@@ -30,6 +30,9 @@
 // Integer adds are native shared-memory atomics and do not depend on their
 // order, so these sums are bit-reproducible; the F-knot sums (FP64 atomics,
 // four per atom) are reproducible to rounding.
+#include <climits>
+#include <type_traits>
+
 #include "k_pair.cuh"
 
 namespace mdk {
@@ -84,26 +87,28 @@ struct Fx64 {
     if (old + vl < old) vh += 1;
     if (vh != 0) atomicAdd(hi + slot, vh);
   }
-  __device__ __forceinline__ void add(int slot, double w, bool) const {
+  template <bool WIDE>
+  __device__ __forceinline__ void add(int slot, double w) const {
     const long long v = __double2ll_rn(w);
     add(slot, (unsigned)v, (int)(v >> 32));
   }
   // A float rounded to 64 bits without the conversion to int64, which runs on
   // GB300's FP64 pipe (16 cycles of an SM per warp; 8 conversions a pair kept
   // that pipe 89% busy): the high word by an FMA at 1.5 2^23 (|w| < 2^53;
-  // wide: terms may be larger, see k_adj_scale), the exact rest (at most 2^31
+  // WIDE: terms may be larger, see k_adj_scale), the exact rest (at most 2^31
   // in magnitude; +2^31 itself, a tie, saturates and is put right) to 32 bits.
-  // k_adj_pair on the 143,460-atom cold-curve batch 243 -> 183 us.
-  __device__ __forceinline__ void add(int slot, float w, bool wide) const {
-    if (wide) {
+  // VJP of the 143,460-atom cold-curve batch 373 -> 318 us (312 with ties one
+  // unit off).
+  template <bool WIDE>
+  __device__ __forceinline__ void add(int slot, float w) const {
+    if constexpr (WIDE) {
       const long long v = __float2ll_rn(w);
       add(slot, (unsigned)v, (int)(v >> 32));
       return;
     }
     const float m = fmaf(w, 0x1p-32f, 12582912.0f);
-    const float rest = fmaf(m - 12582912.0f, -0x1p32f, w);
-    const int vl = __float2int_rn(rest);
-    add(slot, (unsigned)vl + (rest == 0x1p31f ? 1u : 0u),
+    const int vl = __float2int_rn(fmaf(m - 12582912.0f, -0x1p32f, w));
+    add(slot, (unsigned)vl + (vl == INT_MAX ? 1u : 0u),  // no float below 2^31 rounds to it
         __float_as_int(m) - 0x4B400000 + (vl >> 31));
   }
   __device__ __forceinline__ long long get(int slot) const {
@@ -113,14 +118,13 @@ struct Fx64 {
 
 // fixed-point add of cv * (value weights) + cd * (derivative weights) to the
 // slots (y_k, M_k, y_{k+1}, M_{k+1}) = 2k .. 2k + 3
-template <class R>
-__device__ __forceinline__ void scatter_fx(const Fx64 &h, bool wide, int k, R S, R a0, R a1, R a2,
-                                           R a3) {
+template <bool WIDE, class R>
+__device__ __forceinline__ void scatter_fx(const Fx64 &h, int k, R S, R a0, R a1, R a2, R a3) {
   // S is a power of two, so the products are exact
-  h.add(2 * k, a0 * S, wide);
-  h.add(2 * k + 1, a1 * S, wide);
-  h.add(2 * k + 2, a2 * S, wide);
-  h.add(2 * k + 3, a3 * S, wide);
+  h.add<WIDE>(2 * k, a0 * S);
+  h.add<WIDE>(2 * k + 1, a1 * S);
+  h.add<WIDE>(2 * k + 2, a2 * S);
+  h.add<WIDE>(2 * k + 3, a3 * S);
 }
 
 // add a block's shared histogram to the global one (zeros skipped)
@@ -313,7 +317,7 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_pair(Sys s, EAMParams ep, Adj
   for (int q = threadIdx.x; q < 8 * ep.nr; q += blockDim.x) w[q] = 0u;
   __syncthreads();
   const R S = (R)__longlong_as_double(a.aux[4]);
-  const bool wide = a.aux[5] != 0;
+  const bool wide = sizeof(R) == 4 && a.aux[5] != 0;
   const int N = s.st->N;
   const size_t Nc = s.N_cap;
   const V *__restrict__ pg = (const V *)s.pg[a.cur];
@@ -322,7 +326,8 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_pair(Sys s, EAMParams ep, Adj
   const R rc2 = sizeof(R) == 8 ? (R)ep.rc2 : (R)ep.rc2f;
   const R inv_dr = sizeof(R) == 8 ? (R)ep.inv_dr : (R)ep.inv_drf;
   const int kmax = ep.nr - 2;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+  auto pairs_of = [&](const int i, auto wide_terms) {
+    constexpr bool WIDE = decltype(wide_terms)::value;
     const V pi = GP::ld(pg + i);
     const uint32_t inf = GP::info(pi);
     const V gi = GP::ld(gq + i);
@@ -362,13 +367,19 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_pair(Sys s, EAMParams ep, Adj
             const R gd = (gix * dx + giy * dy + giz * dz) * inv_r;
             const R cp = gd * inv_dr;                    // phi': (gF_i . d^) / h
             const R cr = gd * (fpi + q.fp) * inv_dr;     // rho': times F'_i + F'_j
-            scatter_fx<R>(hp, wide, kk, S, half_gE * w[0] + cp * dw[0], half_gE * w[1] + cp * dw[1],
+            scatter_fx<WIDE, R>(hp, kk, S, half_gE * w[0] + cp * dw[0], half_gE * w[1] + cp * dw[1],
                           half_gE * w[2] + cp * dw[2], half_gE * w[3] + cp * dw[3]);
-            scatter_fx<R>(hr, wide, kk, S, lam * w[0] + cr * dw[0], lam * w[1] + cr * dw[1],
+            scatter_fx<WIDE, R>(hr, kk, S, lam * w[0] + cr * dw[0], lam * w[1] + cr * dw[1],
                           lam * w[2] + cr * dw[2], lam * w[3] + cr * dw[3]);
           }
         },
         [] {});
+  };
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+    if (wide)
+      pairs_of(i, std::true_type());
+    else
+      pairs_of(i, std::false_type());
   }
   __syncthreads();
   flush(hp, a.acc_phi, ep.nr);

@@ -24,9 +24,9 @@ __global__ void k(const float *x, long long *o, int n, int wide) {
   hi[t] = 0;
   const mdk::Fx64 h{lo, hi};
   if (i >= n) return;
-  h.add(t, x[i], wide != 0);
+  wide ? h.add<true>(t, x[i]) : h.add<false>(t, x[i]);
   o[i] = h.get(t);
-  h.add(t, -0.75f * x[i], wide != 0);
+  wide ? h.add<true>(t, -0.75f * x[i]) : h.add<false>(t, -0.75f * x[i]);
   o[n + i] = h.get(t);
 }
 extern "C" int run(const float *x, long long *o, int n, int wide) {
