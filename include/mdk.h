@@ -628,7 +628,10 @@ int mdk_get_list_kind(const mdk_ctx *ctx, int *kind);
  * step nor the last step of the call) as one CUDA graph -- a loop on the device
  * of up to 8 force passes per list check, then the rebuild chain -- captured
  * on first use and re-captured whenever a parameter it baked in changes
- * (workspace, potential, launch shape, dt, window...).  Steps taken while mdk_profile records run without graphs.
+ * (workspace, potential, launch shape, dt, window...).  The chain after a first
+ * kick or a thermo step becomes a graph of its own when it is met again; that
+ * one holds neither dt nor the potential.  Steps taken while mdk_profile records
+ * run without graphs.
  */
 int mdk_set_graphs(mdk_ctx *ctx, int enable);
 
